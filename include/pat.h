@@ -113,18 +113,18 @@ int pat_plan_ng(pat_plan plan);
 
 /* Kernel variants of a plan.  Grid sides with a compiled two-level FFT
  * (108, 144, 180, 200, 240, 300 = N1 x N2) have fixed-size variants (eight
- * for 108-240, eleven for 300), all one launch per pass:
- *   0  column and velocity passes on the N1 x N2 factorisation, density
- *      passes on N2 x N1 (4 rows / 4 spectral columns per CTA); the column
- *      passes of the forward sweep, which runs alone on the GPU, take 8
- *      columns per CTA;
+ * for 108-240, eleven for 300).  Variant 0, the default, is the split-axis
+ * step, three launches per time step on the lines of the half spectra along
+ * each axis; the others are the four-pass step, one launch per pass:
  *   1  all passes N1 x N2, 4 rows / 4 columns per CTA;
  *   2  all passes N1 x N2, 8 rows / 2 columns per CTA;
  *   3  as 1 with the row passes' state staged in shared memory by TMA bulk
  *      copies instead of registers;
  *   4  all passes N2 x N1, 4 rows / 4 columns per CTA;
- *   5  as 0 with 8 rows per CTA in the row passes;
- *   6  as 0 with the segment recompute's row passes (which share the GPU
+ *   5  column and velocity passes on the N1 x N2 factorisation, density
+ *      passes on N2 x N1, 8 rows per CTA in the row passes, 8 columns in the
+ *      forward sweep's column passes (which run alone on the GPU), else 4;
+ *   6  as 5 with 4 rows per CTA and the segment recompute's row passes (which share the GPU
  *      with the adjoint) staged by TMA as in 3, so that they need fewer
  *      registers;
  *   7  (108-240) as 5 with column passes that form their multipliers where
@@ -135,7 +135,9 @@ int pat_plan_ng(pat_plan plan);
  *   9  (300) as 5 with 4-column tiles in the forward sweep's column passes;
  *   10 (300) as 5 with the column passes of 7 (108-240).
  * Every side also has the generic shared-memory Stockham passes (variant
- * -1).  All variants compute the same scheme.  A new plan uses variant 0
+ * -1); on sides without variants -1 is the split-axis step where it is
+ * compiled (72, 80, 90, 96, 100, 120, 128, 150, 160, 192, 216, 250, 256, 270,
+ * 288, 320, 324, 360, 384, 400).  All variants compute the same scheme.  A new plan uses variant 0
  * when it exists, else -1.  pat_plan_variants returns the number of
  * fixed-size variants; pat_plan_set_variant selects one (PAT_EINVAL if it
  * does not exist); pat_plan_variant returns the current one. */
@@ -472,7 +474,11 @@ int pat_time_interp(const float* d_y, float* d_out, int K, int nt_src, int nt_ds
 #define PAT_K_COL_SUM 5       /* column pass, two in, one out (adjoint D) */
 #define PAT_K_ROW_ADJ_RHO 6   /* adjoint density row pass (incl. scatter, dJ/dc) */
 #define PAT_K_ROW_ADJ_U 7     /* adjoint velocity row pass */
-#define PAT_K_LAST 7
+/* passes of the split-axis step (pat_plan_set_variant), forward and adjoint alike */
+#define PAT_K_LINES 8         /* lines pass (velocity and density updates of both axes) */
+#define PAT_K_TO_LINES 9      /* real fields to lines (pressure, samples; adjoint: dJ/dc) */
+#define PAT_K_TO_REAL 10      /* lines to real fields (adjoint: sensor source) */
+#define PAT_K_LAST 10
 
 /* Total number of kernels this library has launched in the process. */
 unsigned long long pat_kernel_launches(void);

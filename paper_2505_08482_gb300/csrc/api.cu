@@ -47,6 +47,7 @@ size_t state_bytes(const pat_plan_s* p) { return 4 * size_t(p->K) * p->ng * p->n
 
 // forward steps n0 .. n1-1; p^{n+1} into hist slot n+1-hbase when hist and n+1 >= hbase
 int run_steps(const Launch& L, const Ws& w, int n0, int n1, float* y, float* hist, int hbase) {
+    if (L.split) return split_steps(L, w, n0, n1, y, hist, hbase, nullptr);
     for (int n = n0; n < n1; ++n) {
         const bool h = hist && n + 1 >= hbase;
         RC(step(L, w, n, y, h ? hist : nullptr, n + 1 - hbase));
@@ -57,9 +58,9 @@ int run_steps(const Launch& L, const Ws& w, int n0, int n1, float* y, float* his
 }  // namespace
 
 int pat::forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y, const Ws& w, bool keep,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool allow_split) {
     NvtxRange nv("pat forward sweep");
-    Launch L{p, st, true};
+    Launch L{p, st, true, false, allow_split ? p->split : nullptr};
     RC(launch_medium(L, c, w.cg));
     PAT_CUDA(cudaMemsetAsync(y, 0, size_t(p->K) * p->nt * p->m * sizeof(float), st));
     PAT_CUDA(cudaMemsetAsync(w.flag + 1, 0, sizeof(int), st));   // bounded-wait status of this call
@@ -70,6 +71,10 @@ int pat::forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y,
     if (p->cluster && p->clops)      // one cluster per data set for the whole sweep, state on chip
         return launch_forward_cluster(L, w, p0, nullptr, 0, p->nt - 1, y, hlast, last0, keep ? w.ckpt : nullptr,
                                       w.ux);
+    if (L.split) {                   // three launches per step (ksplit.cuh)
+        RC(split_start(L, w, p0, y, (keep && last0 == 0) ? hlast : nullptr, 0));
+        return split_steps(L, w, 0, p->nt - 1, y, hlast, last0, keep ? w.ckpt : nullptr);
+    }
     RC(launch_row_rho(L, w, 1, p0, y, 0, (keep && last0 == 0) ? hlast : nullptr, 0));
     // segments of s steps with the state copied at their starts (one segment without checkpoints)
     const int seg = keep ? p->s_eff : p->nt;
@@ -94,7 +99,7 @@ namespace {
 
 // recompute segment j's pressure history into its buffer (on stream st)
 int recompute(pat_plan_s* p, const float* p0, const Ws& w, int j, cudaStream_t st) {
-    Launch L{p, st, false, true};
+    Launch L{p, st, false, true, p->split};
     const size_t f = size_t(p->K) * p->ng * p->ng;
     const int n0 = j * p->s_eff;
     const int n1 = std::min(n0 + p->s_eff, p->nt) - 1;
@@ -102,6 +107,11 @@ int recompute(pat_plan_s* p, const float* p0, const Ws& w, int j, cudaStream_t s
     if (p->cluster && p->clops)   // from the checkpoint (or p0) on chip, storing p^n of the segment
         return launch_forward_cluster(L, w, p0, j == 0 ? nullptr : w.ckpt + size_t(j - 1) * 4 * f, n0, n1, nullptr,
                                       h, n0, nullptr, nullptr);
+    if (L.split) {
+        RC(j == 0 ? split_start(L, w, p0, nullptr, h, 0)
+                  : split_enter(L, w, w.ckpt + size_t(j - 1) * 4 * f, n0, nullptr, h, 0));
+        return split_steps(L, w, n0, n1, nullptr, h, n0, nullptr);
+    }
     if (j == 0) {
         RC(launch_row_rho(L, w, 1, p0, nullptr, 0, h, 0));
     } else {
@@ -115,6 +125,7 @@ int recompute(pat_plan_s* p, const float* p0, const Ws& w, int j, cudaStream_t s
 // adjoint steps n_hi down to n_lo (first: n_hi is the first adjoint step of the sweep)
 int run_adj(const Launch& L, const Ws& w, const float* r, int n_hi, int n_lo, bool first, const float* h, int hbase,
             float sg, float sd) {
+    if (L.split) return split_adjoint(L, w, r, n_hi, n_lo, first, h, hbase);
     for (int n = n_hi; n >= n_lo; --n) {
         RC(launch_row_adj_rho(L, w, (first && n == n_hi) ? 1 : 0, r, n, h, n - hbase));
         RC(launch_col(L, w.A2, w.B2, 1, 0, sg));
@@ -130,9 +141,15 @@ int run_adj(const Launch& L, const Ws& w, const float* r, int n_hi, int n_lo, bo
 int reverse_sweep(pat_plan_s* p, const float* p0, const float* r, float* grad_p0, float* grad_c, const Ws& w,
                   bool hist_last_valid, cudaStream_t st) {
     NvtxRange nv("pat reverse sweep");
-    Launch L{p, st};
+    Launch L{p, st, false, false, p->split};
     const size_t f = size_t(p->K) * p->ng * p->ng;
-    PAT_CUDA(cudaMemsetAsync(w.ubx, 0, 4 * f * sizeof(float), st));
+    if (L.split) {
+        const size_t lines = 2 * size_t(p->K) * p->hc * p->ng * sizeof(float2);
+        PAT_CUDA(cudaMemsetAsync(w.lub, 0, lines, st));
+        PAT_CUDA(cudaMemsetAsync(w.lrb, 0, lines, st));
+    } else {
+        PAT_CUDA(cudaMemsetAsync(w.ubx, 0, 4 * f * sizeof(float), st));
+    }
     PAT_CUDA(cudaMemsetAsync(w.cbar, 0, size_t(p->K) * p->n * p->n * sizeof(float), st));
     const float sg = float(p->g.dt * p->g.rho0 / (double(p->ng) * p->ng));   // dt rho0 G t
     const float sd = float(p->g.dt / p->g.rho0 / (double(p->ng) * p->ng));   // dt/rho0 D t'
@@ -165,6 +182,10 @@ int reverse_sweep(pat_plan_s* p, const float* p0, const float* r, float* grad_p0
             RC(recompute(p, p0, w, j - 2, R));
             PAT_CUDA(cudaEventRecord(p->ev_rec[(j - 2) & 1], R));
         }
+    }
+    if (L.split) {
+        RC(split_adjoint_final(L, w, have_q, r, p0, grad_p0));
+        return launch_reduce_cbar(L, w, grad_c);
     }
     RC(launch_row_adj_final1(L, w, have_q ? 0 : 1, r, grad_p0));
     const float s0 = float(-0.5 * p->g.dt / p->g.rho0 / (double(p->ng) * p->ng));
@@ -337,6 +358,7 @@ extern "C" int pat_plan_autotune(pat_plan p, void* ws, size_t ws_bytes, double* 
     for (int v = -1; v < nv && rc == PAT_OK; ++v) {
         rc = select_variant(p, v);
         if (rc != PAT_OK) break;
+        L.split = p->split;
         rc = run_steps(L, w, 1, 4, nullptr, nullptr, 0);   // first launches of the variant's kernels
         if (rc != PAT_OK) break;
         // the median of kSamples timings, so that one disturbed sample cannot decide the choice

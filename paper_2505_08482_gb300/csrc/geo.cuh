@@ -13,7 +13,10 @@ struct Geo {
     int ng, hc, hp, n, P, K, nt, m, s_eff;   // hp: row pitch of a spectrum (>= hc)
     FftDesc fft;
     const float2* tw;
+    const float2* twA;   // per-layout twiddles of the split-axis passes (fft2l.cuh), or null
+    const float2* twB;
     const float* kappa_t;
+    const float* kd;
     const float2* fx;
     const float2* fy;
     const float* a_cell;
@@ -30,7 +33,7 @@ inline Geo geo(const pat_plan_s* p) {
     g.ng = p->ng; g.hc = p->hc; g.hp = p->hp; g.n = p->n; g.P = p->P; g.K = p->K; g.nt = p->nt; g.m = p->m;
     g.s_eff = p->s_eff;
     g.fft = p->fft;
-    g.tw = p->t.tw; g.kappa_t = p->t.kappa_t; g.fx = p->t.fx; g.fy = p->t.fy;
+    g.tw = p->t.tw; g.twA = p->t.twA; g.twB = p->t.twB; g.kappa_t = p->t.kappa_t; g.kd = p->t.kd; g.fx = p->t.fx; g.fy = p->t.fy;
     g.a_cell = p->t.a_cell; g.a_stag = p->t.a_stag;
     g.srow = p->t.srow; g.sent = p->t.sent; g.sentw = p->t.sentw;
     g.kinst = p->t.kinst;

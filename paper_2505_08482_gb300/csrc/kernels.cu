@@ -579,8 +579,17 @@ int configure_kernels(pat_plan_s* p) {
 }
 
 int select_variant(pat_plan_s* p, int variant) {
+    // the split-axis passes are variant 0 of the sides that have variants and the only form of the
+    // others (which report the generic variant -1)
+    const SplitOps* sp = split_ops_for(p->ng);
+    if (variant > 0 || (variant < 0 && fixed_variants(p->ng) > 0)) sp = nullptr;
+    if (sp) {
+        const int rc = split_configure(sp);
+        if (rc != PAT_OK) return rc;
+    }
     if (variant < 0) {
         p->fast = nullptr;
+        p->split = sp;
         p->variant = -1;
         return PAT_OK;
     }
@@ -592,6 +601,7 @@ int select_variant(pat_plan_s* p, int variant) {
     int rc = f->configure();
     if (rc != PAT_OK) return rc;
     p->fast = f;
+    p->split = sp;
     p->variant = variant;
     return PAT_OK;
 }

@@ -54,10 +54,10 @@ extern "C" int pat_forward_noalloc(pat_plan p, const float* c, const float* p0, 
         pat::set_error("pat_forward_noalloc: null argument");
         return PAT_EINVAL;
     }
-    if (p->ws_fwd > size_t(PAT_NOALLOC_SCRATCH_BYTES)) {
+    if (p->ws_fwd_passes > size_t(PAT_NOALLOC_SCRATCH_BYTES)) {
         pat::set_error("pat_forward_noalloc: this plan needs %zu bytes of scratch but the static scratch holds %d "
                        "bytes (reduce K or the grid, or use pat_forward with a workspace)",
-                       p->ws_fwd, PAT_NOALLOC_SCRATCH_BYTES);
+                       p->ws_fwd_passes, PAT_NOALLOC_SCRATCH_BYTES);
         return PAT_EINVAL;
     }
     int rc = check_device(p, "pat_forward_noalloc");
@@ -68,7 +68,9 @@ extern "C" int pat_forward_noalloc(pat_plan p, const float* c, const float* p0, 
     // the forward sweep writes every scratch region it reads before reading it,
     // so nothing left by an earlier call needs clearing
     pat::Ws w = pat::resolve(p, scratch, false);
-    rc = pat::forward_sweep(p, c, p0, y, w, false, static_cast<cudaStream_t>(stream));
+    // the split-axis passes where their larger state fits the array too, else the four-pass step
+    rc = pat::forward_sweep(p, c, p0, y, w, false, static_cast<cudaStream_t>(stream),
+                            p->ws_fwd <= size_t(PAT_NOALLOC_SCRATCH_BYTES));
     if (rc != PAT_OK) return rc;
     p->hist_valid_ws = nullptr;
     return PAT_OK;

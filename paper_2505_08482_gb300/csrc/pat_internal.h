@@ -19,6 +19,7 @@ namespace pat {
 struct FixedOps;
 struct SweepOps;
 struct ClusterOps;
+struct SplitOps;
 
 // NVTX range on the host timeline for the lifetime of the object (profilers show the library's
 // calls, sweeps and multigrid levels by name; without a profiler attached it costs a branch)
@@ -40,7 +41,10 @@ int cuda_fail(cudaError_t e, const char* where);
 // Device tables of one plan (all built in FP64 on the host, stored FP32).
 struct Tables {
     float2* tw;        // [ng] exp(-2 pi i q / ng)
+    float2* twA;       // [ng] each: the twiddles of the split-axis passes in the order of their two
+    float2* twB;       // transform steps (null: no split-axis passes for this side)
     float* kappa_t;    // [hc][ng] kappa(kx, ky) at kx * ng + ky
+    float* kd;         // [hc][ng] kappa dt ng^{-3/2}, corrected for the transforms' gain (split-axis passes, or null)
     float2* fx;        // [hc] i kx exp(+i kx dx/2)   (x factor of G; D uses -conj)
     float2* fy;        // [ng] i ky exp(+i ky dx/2)   (y factor of G; D uses -conj)
     float* a_cell;     // [ng] PML factor at cell centres
@@ -59,6 +63,10 @@ struct Ws {
     float2* A; float2* B;                         // spectra [K][ng][hc]
     double* J; double* part; int* flag;           // objective per instance, partial sums [K][32], flag
     int* queue;                                   // persistent sweep: tickets, abort flag, done per data set
+    // the split-axis passes' view of the same memory: lines [2][K][hc][ng] of u, rho and the pressure,
+    // real rho_x, rho_y [2][K][ng][ng]; the adjoint's below
+    float2* lu; float2* lr; float2* la; float* re;
+    float2* lub; float2* lrb; float2* la2; float* re2;
     // gradient only
     float* ckpt;                                  // [nseg-1][4][K][ng][ng]
     float* hist;                                  // [2][K][s_eff][ng][ng] pressure history (two segments)
@@ -80,6 +88,7 @@ struct pat_plan_s {
     int ninst;         // instances sharing the grid; K counts the data sets of all of them
     pat::FftDesc fft;
     const pat::FixedOps* fast;   // fixed-size passes for this grid side (nullptr: generic Stockham)
+    const pat::SplitOps* split;  // split-axis passes in use (nullptr: the four-pass step of `fast`)
     const pat::SweepOps* sweep;  // persistent forward sweep of this grid side (nullptr: none)
     bool persistent;             // forward sweeps run as one persistent launch
     const pat::ClusterOps* clops;   // cluster-resident stepping of this grid side (nullptr: none)
@@ -92,9 +101,11 @@ struct pat_plan_s {
     pat::Tables t;
     int nent;
     size_t ws_fwd, ws_grad;
+    size_t ws_fwd_passes;   // forward workspace of the four-pass step alone
     // layout offsets (bytes)
     size_t o_state, o_cg, o_A, o_B, o_J, o_part, o_flag, o_queue;
     size_t o_ckpt, o_hist, o_adj, o_A2, o_B2, o_cbar, o_resid, o_ypred;
+    size_t o_lu, o_lr, o_la, o_re, o_lub, o_lrb, o_la2, o_re2;   // split-axis views
     // host bookkeeping: the workspace whose history holds the last segment
     const void* hist_valid_ws;
     int device;
@@ -139,6 +150,7 @@ struct Launch {
     cudaStream_t st;
     bool solo = false;        // no other stream of this call runs beside it (the forward sweep)
     bool recompute = false;   // the segment recompute, which runs beside the adjoint
+    const SplitOps* split = nullptr;   // split-axis passes instead of the four-pass step
 };
 
 int configure_kernels(pat_plan_s* p);
@@ -177,10 +189,29 @@ int launch_residual(const Launch& L, const Ws& w, const float* ypred, const floa
 int launch_forward_cluster(const Launch& L, const Ws& w, const float* p0, const float* state, int n0, int n1,
                            float* y, float* hist, int hist_base, float* ckpt, float* state_out);
 
+// ---- split-axis passes (split.cu) ----
+// the initial pass from p0: rho lines, pressure lines, samples of level 0 (y, hist may be null)
+int split_start(const Launch& L, const Ws& w, const float* p0, float* y, float* hist, int hist_slot);
+// re-enter at a level from the real state [4][K][ng][ng] (u_x, u_y, rho_x, rho_y): lines of u and rho
+// (after_copy: the state may have been written by a copy), then the samples and pressure lines of that level
+int split_enter(const Launch& L, const Ws& w, const float* state, int level, float* y, float* hist, int hist_slot);
+// forward steps n0 .. n1-1; p^{n+1} into slot n+1-hbase of hist when hist and n+1 >= hbase; ckpt (or
+// null): the real state at every level that is a multiple of s, from which the sweep itself goes on,
+// so that a recompute from the checkpoint repeats it bit for bit
+int split_steps(const Launch& L, const Ws& w, int n0, int n1, float* y, float* hist, int hbase, float* ckpt);
+// adjoint steps n_hi .. n_lo (first: n_hi opens the sweep), and the transposes of the initial condition
+int split_adjoint(const Launch& L, const Ws& w, const float* r, int n_hi, int n_lo, bool first, const float* h,
+                  int hbase);
+int split_adjoint_final(const Launch& L, const Ws& w, bool have_q, const float* r, const float* p0, float* grad_p0);
+const SplitOps* split_ops_for(int ng);   // nullptr: no split-axis passes for this grid side
+bool split_factors(int ng, int* n1, int* n2, double* gain);   // gain: SplitOps::pair_gain
+int split_configure(const SplitOps* ops);
+
 // ---- api.cu internals ----
 // Forward sweep into y [K][nt][m] with workspace regions w (checkpoints kept if keep).
+// allow_split = false: the four-pass step (a workspace too small for the split-axis passes).
 int forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y, const Ws& w, bool keep,
-                  cudaStream_t st);
+                  cudaStream_t st, bool allow_split = true);
 // used by the reconstruction driver:
 // J only (forward sweep + residual) into *J_dev; workspace of PAT_WS_GRADIENT size.
 int objective(pat_plan_s* p, const float* c, const float* p0, const float* ymeas, const float* wts, double* J_dev,

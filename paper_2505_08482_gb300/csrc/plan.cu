@@ -85,7 +85,15 @@ Ws resolve(const pat_plan_s* p, void* base, bool grad) {
     w.part = reinterpret_cast<double*>(b + p->o_part);
     w.flag = reinterpret_cast<int*>(b + p->o_flag);
     w.queue = reinterpret_cast<int*>(b + p->o_queue);
+    w.lu = reinterpret_cast<float2*>(b + p->o_lu);
+    w.lr = reinterpret_cast<float2*>(b + p->o_lr);
+    w.la = reinterpret_cast<float2*>(b + p->o_la);
+    w.re = reinterpret_cast<float*>(b + p->o_re);
     if (grad) {
+        w.lub = reinterpret_cast<float2*>(b + p->o_lub);
+        w.lrb = reinterpret_cast<float2*>(b + p->o_lrb);
+        w.la2 = reinterpret_cast<float2*>(b + p->o_la2);
+        w.re2 = reinterpret_cast<float*>(b + p->o_re2);
         w.ckpt = reinterpret_cast<float*>(b + p->o_ckpt);
         w.hist = reinterpret_cast<float*>(b + p->o_hist);
         float* ad = reinterpret_cast<float*>(b + p->o_adj);
@@ -102,24 +110,43 @@ Ws resolve(const pat_plan_s* p, void* base, bool grad) {
     return w;
 }
 
+// The four-pass step and the split-axis passes lay their state over the same memory (a plan runs one
+// of them at a time; checkpoints and the pressure history are real fields in both).
 static void layout(pat_plan_s* p) {
     const size_t f = size_t(p->K) * p->ng * p->ng * sizeof(float);
     const size_t spec = size_t(p->K) * p->ng * p->hp * sizeof(float2);
+    const size_t lines = 2 * size_t(p->K) * p->hc * p->ng * sizeof(float2);
+    const bool split = split_ops_for(p->ng) != nullptr;
     size_t o = 0;
-    p->o_state = o; o = align256(o + 4 * f);
     p->o_cg = o; o = align256(o + size_t(p->ninst) * p->ng * p->ng * sizeof(float));
-    p->o_A = o; o = align256(o + spec);
-    p->o_B = o; o = align256(o + spec);
     p->o_J = o; o = align256(o + size_t(p->ninst) * sizeof(double));
     p->o_part = o; o = align256(o + size_t(p->K) * kResidBlocks * sizeof(double));
     p->o_flag = o; o = align256(o + 4 * sizeof(int));
     p->o_queue = o; o = align256(o + (size_t(p->K) + 2) * sizeof(int));
+    const size_t fwd = o;
+    p->o_state = o; o = align256(o + 4 * f);
+    p->o_A = o; o = align256(o + spec);
+    p->o_B = o; o = align256(o + spec);
+    p->ws_fwd_passes = o;
+    size_t q = fwd;
+    p->o_lu = q; q = align256(q + lines);
+    p->o_lr = q; q = align256(q + lines);
+    p->o_la = q; q = align256(q + lines);
+    p->o_re = q; q = align256(q + 2 * f);
+    if (split) o = std::max(o, q);
     p->ws_fwd = o;
     p->o_ckpt = o; o = align256(o + size_t(std::max(p->nseg - 1, 0)) * 4 * f);
     p->o_hist = o; o = align256(o + size_t(p->nseg > 1 ? 2 : 1) * p->K * p->s_eff * p->ng * p->ng * sizeof(float));
+    const size_t adj = o;
     p->o_adj = o; o = align256(o + 4 * f);
     p->o_A2 = o; o = align256(o + spec);
     p->o_B2 = o; o = align256(o + spec);
+    q = adj;
+    p->o_lub = q; q = align256(q + lines);
+    p->o_lrb = q; q = align256(q + lines);
+    p->o_la2 = q; q = align256(q + lines);
+    p->o_re2 = q; q = align256(q + 2 * f);
+    if (split) o = std::max(o, q);
     p->o_cbar = o; o = align256(o + size_t(p->K) * p->n * p->n * sizeof(float));
     const size_t tr = size_t(p->K) * p->nt * p->m * sizeof(float);
     p->o_resid = o; o = align256(o + tr);
@@ -266,6 +293,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     p->s_eff = std::min(ckpt_every, g->nt);
     p->nseg = (g->nt + p->s_eff - 1) / p->s_eff;
     p->hist_valid_ws = nullptr;
+    p->split = nullptr;
     p->sweep = nullptr;
     p->persistent = false;
     p->clops = nullptr;
@@ -290,6 +318,17 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
         double a = -2.0 * PI * q / ng;
         tw[q] = make_float2(float(std::cos(a)), float(std::sin(a)));
     }
+    // the same twiddles in the order in which the two transform steps of the split-axis passes read them
+    std::vector<float2> twA, twB;
+    int f1 = 0, f2 = 0;
+    double gain = 0.0;
+    const bool split = split_factors(ng, &f1, &f2, &gain);
+    if (split) {
+        twA.resize(ng);
+        twB.resize(ng);
+        for (int a = 0; a < f1; ++a)
+            for (int b = 0; b < f2; ++b) twA[a * f2 + b] = twB[b * f1 + a] = tw[(a * b) % ng];
+    }
     auto gfac = [&](double k, bool nyq) {
         // i k exp(+i k dx/2); real at the Nyquist wavenumber
         double c = std::cos(0.5 * k * dx), s = std::sin(0.5 * k * dx);
@@ -299,12 +338,16 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     };
     for (int i = 0; i < p->hc; ++i) fx[i] = gfac(k1[i], i == ng / 2);
     for (int i = 0; i < ng; ++i) fy[i] = gfac(k1[i], i == ng / 2);
-    std::vector<float> kap(size_t(p->hc) * ng);
+    std::vector<float> kap(size_t(p->hc) * ng), kd(split ? kap.size() : 0);
+    // three transform pairs per step share the correction between G and D
+    const double kscale = dt / (ng * std::sqrt(double(ng))) * std::pow(1.0 + gain, -1.5);
     for (int kx = 0; kx < p->hc; ++kx)
         for (int ky = 0; ky < ng; ++ky) {
             double kk = std::sqrt(k1[kx] * k1[kx] + k1[ky] * k1[ky]);
             double a = 0.5 * g->c_ref * kk * dt;
-            kap[size_t(kx) * ng + ky] = float(a == 0.0 ? 1.0 : std::sin(a) / a);
+            const double v = a == 0.0 ? 1.0 : std::sin(a) / a;
+            kap[size_t(kx) * ng + ky] = float(v);
+            if (split) kd[size_t(kx) * ng + ky] = float(kscale * v);
         }
     std::vector<float> ac(ng), as(ng);
     for (int i = 0; i < ng; ++i) {
@@ -354,6 +397,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     // ---- one device allocation for all tables ----
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
+    size_t o_kd = take(kd.size() * sizeof(float)), o_ta = take(twA.size() * sizeof(float2)), o_tb = take(twB.size() * sizeof(float2));
     size_t o_tw = take(ng * sizeof(float2)), o_k = take(kap.size() * sizeof(float));
     size_t o_fx = take(p->hc * sizeof(float2)), o_fy = take(ng * sizeof(float2));
     size_t o_ac = take(ng * sizeof(float)), o_as = take(ng * sizeof(float));
@@ -368,6 +412,9 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     }
     char* d = static_cast<char*>(p->dev);
     p->t.tw = reinterpret_cast<float2*>(d + o_tw);
+    p->t.kd = split ? reinterpret_cast<float*>(d + o_kd) : nullptr;
+    p->t.twA = twA.empty() ? nullptr : reinterpret_cast<float2*>(d + o_ta);
+    p->t.twB = twB.empty() ? nullptr : reinterpret_cast<float2*>(d + o_tb);
     p->t.kappa_t = reinterpret_cast<float*>(d + o_k);
     p->t.fx = reinterpret_cast<float2*>(d + o_fx);
     p->t.fy = reinterpret_cast<float2*>(d + o_fy);
@@ -380,6 +427,9 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     p->t.kfirst = reinterpret_cast<int*>(d + o_kf);
     struct Cp { void* dst; const void* src; size_t n; } cps[] = {
         {p->t.tw, tw.data(), ng * sizeof(float2)},
+        {p->t.twA, twA.data(), twA.size() * sizeof(float2)},
+        {p->t.kd, kd.data(), kd.size() * sizeof(float)},
+        {p->t.twB, twB.data(), twB.size() * sizeof(float2)},
         {p->t.kappa_t, kap.data(), kap.size() * sizeof(float)},
         {p->t.fx, fx.data(), p->hc * sizeof(float2)},
         {p->t.fy, fy.data(), ng * sizeof(float2)},
@@ -392,7 +442,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
         {p->t.kfirst, kfirst.data(), (ninst + 1) * sizeof(int)},
     };
     for (const Cp& c : cps)
-        if (e == cudaSuccess) e = cudaMemcpy(c.dst, c.src, c.n, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && c.n > 0) e = cudaMemcpy(c.dst, c.src, c.n, cudaMemcpyHostToDevice);
     // copies from pageable memory may still be in flight when cudaMemcpy returns, and the
     // caller's non-blocking streams are not ordered after the legacy stream: wait for them
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
