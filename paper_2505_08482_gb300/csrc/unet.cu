@@ -8,11 +8,12 @@
 // (nearest, 2x), concatenates the encoder output of level l, and applies two
 // 3x3 convolutions with ReLU and F 2^l channels; a 1x1 convolution gives the
 // single output channel.  Activations are BF16 NHWC with channel counts
-// padded to multiples of 8; every convolution is im2col + one tensor-core
-// GEMM (forward), im2col of the output gradient with flipped taps + GEMM
-// (data gradient) and a split-K GEMM of transposed operands (weight
-// gradient), FP32 accumulation throughout; parameters are FP32 masters with
-// BF16 copies, updated by Adam.
+// padded to multiples of 8; the 3x3 convolutions, their data and weight
+// gradients are implicit GEMMs on the tensor cores (unet_conv.cu) where the
+// channel counts are multiples of 16, else im2col + one GEMM (forward, data
+// gradient) and a split-K GEMM of transposed operands (weight gradient), as
+// always on the warp-level path; FP32 accumulation throughout; parameters are
+// FP32 masters with BF16 copies, updated by Adam.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -56,7 +57,10 @@ struct pat_unet_s {
     size_t nparam = 0, nweight_bf = 0;
     float *param = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16* wbf = nullptr;        // bf16 weights (GEMM B operands)
-    __nv_bfloat16* wt = nullptr;         // scratch: transposed weights for the data gradient
+    __nv_bfloat16* wt = nullptr;         // bf16 weights with input and output channels exchanged (data gradient)
+    ConvDesc* desc = nullptr;            // device copy of the convolutions' weight places
+    float* bpart = nullptr;              // partial sums of the bias gradients and the head
+    const Conv* col_of = nullptr;        // the convolution whose im2col of the current input `col` holds
     __nv_bfloat16* col = nullptr;        // scratch: im2col / transposes
     __nv_bfloat16* colt = nullptr;
     __nv_bfloat16* dt = nullptr;         // scratch: transposed output gradient
@@ -93,49 +97,55 @@ int net_gemm(pat_unet_s* u, cudaStream_t st, const __nv_bfloat16* A, int lda, co
     return unet_gemm(st, A, lda, B, ldb, M, N, K, bias, relu, C, ldc, out_mode, splitk);
 }
 
-// conv forward: out = ReLU(conv(in) + b) (relu=0 for the final 1x1)
-int conv_fwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16* in, int ldin, int B, void* out,
-             int out_mode, int relu) {
-    const int P = B * c.H * c.W;
-    const __nv_bfloat16* wb = u->wbf + c.wb_off;
-    const float* bias = u->param + c.b_off;
-    if (c.k == 3) {
-        RC(unet_im2col(st, in, u->col, B, c.H, c.W, c.cin, ldin, 0));
-        return net_gemm(u, st, u->col, 9 * c.cin, wb, 9 * c.cin, P, c.cout, 9 * c.cin, bias, relu, out, c.cout,
-                         out_mode, 1);
-    }
-    return net_gemm(u, st, in, ldin, wb, c.cin, P, c.cout, c.cin, bias, relu, out, c.cout, out_mode, 1);
+// rows of the im2col buffer: 9 cin channels, padded to whole 16-wide steps of the weight gradient
+int col_pitch(int cin) { return (9 * cin + 15) / 16 * 16; }
+
+int make_col(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16* in, int ldin, int B) {
+    if (u->col_of == &c) return PAT_OK;
+    u->col_of = &c;
+    return unet_im2col(st, in, u->col, B, c.H, c.W, c.cin, ldin, 0, col_pitch(c.cin));
 }
 
-// conv backward: given dz = dL/d(pre-activation) [P][cout], accumulate the parameter gradients
-// and (if din) write dL/din [P][cin] (pitch ldin_out)
+// 3x3 convolution forward: out = ReLU(conv(in) + b)
+int conv_fwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16* in, int ldin, int B,
+             __nv_bfloat16* out) {
+    const __nv_bfloat16* wb = u->wbf + c.wb_off;
+    const float* bias = u->param + c.b_off;
+    if (u->gemm_path == 1 && unet_conv_supported(in, ldin, c.cin, c.cout))
+        return unet_conv(st, in, ldin, wb, B, c.H, c.W, c.cin, c.cout, 0, bias, 1, nullptr, out, c.cout, u->status);
+    RC(make_col(u, st, c, in, ldin, B));
+    return net_gemm(u, st, u->col, col_pitch(c.cin), wb, 9 * c.cin, B * c.H * c.W, c.cout, 9 * c.cin, bias, 1, out,
+                    c.cout, 0, 1);
+}
+
+// 3x3 convolution backward: given dz = dL/d(pre-activation) [P][cout], the parameter gradients (dW zeroed by the
+// caller) and (if din) dL/din [P][cin], zero where mask <= 0 (mask: the ReLU output that in is, or null)
 int conv_bwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16* in, int ldin, int B,
-             const __nv_bfloat16* dz, __nv_bfloat16* din) {
-    const int P = B * c.H * c.W;
-    const int K1 = c.k * c.k * c.cin;
+             const __nv_bfloat16* dz, __nv_bfloat16* din, const __nv_bfloat16* mask) {
+    const int P = B * c.H * c.W, K1 = 9 * c.cin;
     float* dW = u->grad + c.w_off;
-    float* db = u->grad + c.b_off;
-    RC(unet_bias_grad(st, dz, db, size_t(P), c.cout, c.cout));
-    // weight gradient: dW[co][k] = sum_p dz[p][co] col[p][k]  (transposed operands, split K over pixels)
-    RC(unet_transpose(st, dz, u->dt, P, c.cout, c.cout));
-    if (c.k == 3) {
-        RC(unet_im2col(st, in, u->col, B, c.H, c.W, c.cin, ldin, 0));
-        RC(unet_transpose(st, u->col, u->colt, P, K1, K1));
-    } else {
-        RC(unet_transpose(st, in, u->colt, P, K1, ldin));
+    RC(unet_bias_grad(st, dz, u->grad + c.b_off, u->bpart, size_t(P), c.cout));
+    if (u->gemm_path == 1 && unet_wgrad_supported(in, ldin, c.cin, c.cout)) {
+        RC(unet_wgrad(st, in, ldin, dz, B, c.H, c.W, c.cin, 9, c.cout, dW, K1, u->status));
+    } else if (u->gemm_path == 1 && unet_wgrad_supported(u->col, col_pitch(c.cin), col_pitch(c.cin), c.cout)) {
+        RC(make_col(u, st, c, in, ldin, B));
+        RC(unet_wgrad(st, u->col, col_pitch(c.cin), dz, B, c.H, c.W, col_pitch(c.cin), 1, c.cout, dW, K1, u->status));
+    } else {   // dW[co][k] = sum_p dz[p][co] col[p][k] from transposed operands, split K over pixels
+        RC(unet_transpose(st, dz, u->dt, P, c.cout, c.cout));
+        RC(make_col(u, st, c, in, ldin, B));
+        RC(unet_transpose(st, u->col, u->colt, P, K1, col_pitch(c.cin)));
+        const int splitk = std::max(1, std::min(64, P / 4096));
+        RC(net_gemm(u, st, u->dt, P, u->colt, P, c.cout, K1, P, nullptr, 0, dW, K1, 2, splitk));
     }
-    PAT_CUDA(cudaMemsetAsync(dW, 0, c.nw() * sizeof(float), st));
-    const int splitk = std::max(1, std::min(64, P / 4096));
-    RC(net_gemm(u, st, u->dt, P, u->colt, P, c.cout, K1, P, nullptr, 0, dW, K1, 2, splitk));
     if (!din) return PAT_OK;
-    // data gradient: din[p][ci] = sum_{tap,co} dz[p - off(tap)][co] W[co][tap][ci]
-    if (c.k == 3) {
-        RC(unet_weight_t(st, u->wbf + c.wb_off, u->wt, c.cout, c.cin));
-        RC(unet_im2col(st, dz, u->col, B, c.H, c.W, c.cout, c.cout, 1));
-        return net_gemm(u, st, u->col, 9 * c.cout, u->wt, 9 * c.cout, P, c.cin, 9 * c.cout, nullptr, 0, din, c.cin,
-                         0, 1);
-    }
-    return PAT_EINVAL;
+    // din[p][ci] = sum_{tap,co} dz[p - off(tap)][co] W[co][tap][ci]
+    const __nv_bfloat16* wt = u->wt + c.wb_off;
+    if (u->gemm_path == 1 && unet_conv_supported(dz, c.cout, c.cout, c.cin))
+        return unet_conv(st, dz, c.cout, wt, B, c.H, c.W, c.cout, c.cin, 1, nullptr, 0, mask, din, c.cin, u->status);
+    u->col_of = nullptr;
+    RC(unet_im2col(st, dz, u->col, B, c.H, c.W, c.cout, c.cout, 1, 9 * c.cout));
+    RC(net_gemm(u, st, u->col, 9 * c.cout, wt, 9 * c.cout, P, c.cin, 9 * c.cout, nullptr, 0, din, c.cin, 0, 1));
+    return mask ? unet_relu_bwd(st, din, mask, size_t(P) * c.cin) : PAT_OK;
 }
 
 // activation indices: enc[l] conv a/b -> 2l, 2l+1; pooled outputs follow; see build()
@@ -161,15 +171,16 @@ Layout layout_of(const pat_unet_s* u) {
     return L;
 }
 
-int forward(pat_unet_s* u, cudaStream_t st, const float* d_in, int B) {
+int forward(pat_unet_s* u, cudaStream_t st, const float* d_in, int B, float* out) {
     Layout L = layout_of(u);
     auto& A = u->acts;
+    u->col_of = nullptr;
     RC(unet_pack_input(st, d_in, A[L.input].y, B, u->in_ch, u->H, u->W, u->cin_pad));
     int ci = 0;
     const Act* prev = &A[L.input];
     for (int l = 0; l < u->levels; ++l) {
-        RC(conv_fwd(u, st, u->convs[ci++], prev->y, prev->C, B, A[L.enc_a[l]].y, 0, 1));
-        RC(conv_fwd(u, st, u->convs[ci++], A[L.enc_a[l]].y, A[L.enc_a[l]].C, B, A[L.enc_b[l]].y, 0, 1));
+        RC(conv_fwd(u, st, u->convs[ci++], prev->y, prev->C, B, A[L.enc_a[l]].y));
+        RC(conv_fwd(u, st, u->convs[ci++], A[L.enc_a[l]].y, A[L.enc_a[l]].C, B, A[L.enc_b[l]].y));
         prev = &A[L.enc_b[l]];
         if (l < u->levels - 1) {
             const Act& pa = A[L.pool[l]];
@@ -178,16 +189,15 @@ int forward(pat_unet_s* u, cudaStream_t st, const float* d_in, int B) {
         }
     }
     for (int d = 0; d < u->levels - 1; ++d) {
-        const int l = u->levels - 2 - d;
         const Act& cat = A[L.dec_cat[d]];
-        const Act& skip = A[L.enc_b[l]];
-        RC(unet_upsample(st, prev->y, cat.y, B, prev->H, prev->W, prev->C, prev->C, cat.C, 0));
-        RC(unet_copy_ch(st, skip.y, cat.y, size_t(B) * skip.H * skip.W, skip.C, skip.C, cat.C, prev->C));
-        RC(conv_fwd(u, st, u->convs[ci++], cat.y, cat.C, B, A[L.dec_a[d]].y, 0, 1));
-        RC(conv_fwd(u, st, u->convs[ci++], A[L.dec_a[d]].y, A[L.dec_a[d]].C, B, A[L.dec_b[d]].y, 0, 1));
+        const Act& skip = A[L.enc_b[u->levels - 2 - d]];
+        RC(unet_concat(st, prev->y, skip.y, cat.y, B, prev->H, prev->W, prev->C, skip.C));
+        RC(conv_fwd(u, st, u->convs[ci++], cat.y, cat.C, B, A[L.dec_a[d]].y));
+        RC(conv_fwd(u, st, u->convs[ci++], A[L.dec_a[d]].y, A[L.dec_a[d]].C, B, A[L.dec_b[d]].y));
         prev = &A[L.dec_b[d]];
     }
-    return conv_fwd(u, st, u->convs[ci], prev->y, prev->C, B, u->out, 1, 0);
+    const Conv& h = u->convs[ci];
+    return unet_head(st, prev->y, u->wbf + h.wb_off, u->param + h.b_off, out, size_t(B) * u->H * u->W, h.cin);
 }
 
 int check_batch(const pat_unet_s* u, int B) {
@@ -277,28 +287,39 @@ extern "C" int pat_unet_create(pat_unet* out, int levels, int base, int in_ch, i
         u->pidx.push_back(p);
     }
     // scratch: the largest im2col (and its transpose) over all convolutions, forward and data gradient
-    size_t colmax = 0, wtmax = 0, dtmax = 0;
+    size_t colmax = 0, dtmax = 0;
+    int cmax = 0;
     for (const Conv& c : u->convs) {
         const size_t P = size_t(max_batch) * c.H * c.W;
-        colmax = std::max(colmax, P * size_t(c.k * c.k) * std::max(c.cin, c.cout));
-        wtmax = std::max(wtmax, c.nw());
+        colmax = std::max(colmax, P * std::max(size_t(c.k * c.k) * std::max(c.cin, c.cout), size_t(col_pitch(c.cin))));
         dtmax = std::max(dtmax, P * size_t(std::max(c.cout, 8)));
+        cmax = std::max(cmax, std::max(c.cin, c.cout));
     }
     u->col_elems = colmax;
     if (rc == PAT_OK) rc = dalloc(u, &u->col, colmax);
     if (rc == PAT_OK) rc = dalloc(u, &u->colt, colmax);
     if (rc == PAT_OK) rc = dalloc(u, &u->dt, dtmax);
-    if (rc == PAT_OK) rc = dalloc(u, &u->wt, std::max<size_t>(wtmax, 8 * 64));
+    if (rc == PAT_OK) rc = dalloc(u, &u->wt, u->nweight_bf);
+    if (rc == PAT_OK) rc = dalloc(u, &u->desc, u->convs.size());
+    if (rc == PAT_OK) rc = dalloc(u, &u->bpart, unet_part_floats(cmax));
     if (rc == PAT_OK) rc = dalloc(u, &u->param, u->nparam);
     if (rc == PAT_OK) rc = dalloc(u, &u->grad, u->nparam);
     if (rc == PAT_OK) rc = dalloc(u, &u->m, u->nparam);
     if (rc == PAT_OK) rc = dalloc(u, &u->v, u->nparam);
     if (rc == PAT_OK) rc = dalloc(u, &u->wbf, u->nweight_bf);
     if (rc == PAT_OK) rc = dalloc(u, &u->out, size_t(max_batch) * H * W);
-    if (rc == PAT_OK) rc = dalloc(u, &u->part, 256);
+    if (rc == PAT_OK) rc = dalloc(u, &u->part, unet_part_blocks());
     if (rc == PAT_OK) rc = dalloc(u, &u->loss, 1);
     if (rc == PAT_OK) rc = dalloc(u, &u->status, 1);
     if (rc == PAT_OK && cudaMemset(u->status, 0, sizeof(int)) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "unet status");
+    if (rc == PAT_OK) {
+        std::vector<ConvDesc> d;
+        for (const Conv& c : u->convs) d.push_back(ConvDesc{c.cin, c.cout, c.k, c.w_off, c.wb_off});
+        // waits for the copy: the caller's streams are not ordered after the legacy stream
+        if (cudaMemcpy(u->desc, d.data(), d.size() * sizeof(ConvDesc), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+            rc = cuda_fail(cudaGetLastError(), "unet weight table");
+    }
     if (rc != PAT_OK) {
         pat_unet_destroy(u);
         return rc;
@@ -334,8 +355,9 @@ extern "C" int pat_unet_param_layout(pat_unet u, int* n_convs, int* h_desc) {
 
 // refresh the bf16 weight copies from the fp32 parameters
 static int sync_bf16(pat_unet_s* u, cudaStream_t st) {
-    for (const Conv& c : u->convs) RC(unet_f32_to_bf16(st, u->param + c.w_off, u->wbf + c.wb_off, c.nw()));
-    return PAT_OK;
+    size_t most = 0;
+    for (const Conv& c : u->convs) most = std::max(most, c.nw());
+    return unet_weights(st, u->param, u->wbf, u->wt, u->desc, int(u->convs.size()), most);
 }
 
 extern "C" int pat_unet_set_params(pat_unet u, const float* d_params, void* stream) {
@@ -359,44 +381,24 @@ extern "C" int pat_unet_forward(pat_unet u, const float* d_in, int B, float* d_o
     if (!u || !d_in || !d_out) { set_error("pat_unet_forward: null argument"); return PAT_EINVAL; }
     RC(check_batch(u, B));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    RC(forward(u, st, d_in, B));
-    PAT_CUDA(cudaMemcpyAsync(d_out, u->out, size_t(B) * u->H * u->W * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    return PAT_OK;
+    return forward(u, st, d_in, B, d_out);
 }
 
 // loss and parameter gradients (into the model's gradient buffer, optionally copied to d_grad)
 static int loss_and_grads(pat_unet_s* u, cudaStream_t st, const float* d_in, const float* d_target, int B) {
-    RC(forward(u, st, d_in, B));
+    for (const Conv& c : u->convs)   // the weight gradient's GEMMs run over the pixels in eights on either path
+        if ((size_t(B) * c.H * c.W) % 8 != 0) {
+            set_error("pat_unet: the gradients need a multiple of 8 pixels on every level (%d x %d x %d)", B, c.H, c.W);
+            return PAT_EINVAL;
+        }
+    RC(forward(u, st, d_in, B, u->out));
     const size_t P = size_t(B) * u->H * u->W;
     const Act& top = u->acts.back();
-    // dL/dout in a bf16 [P][8] buffer (channel 0 used) for the final 1x1 convolution
-    __nv_bfloat16* dout = u->dt;
-    PAT_CUDA(cudaMemsetAsync(dout, 0, P * 8 * sizeof(__nv_bfloat16), st));
-    RC(unet_mse(st, u->out, d_target, dout, P, 8, u->part, u->loss));
-    // final conv (1x1, cin -> 1): gradients by GEMMs on [P][8] operands
+    PAT_CUDA(cudaMemsetAsync(u->grad, 0, u->nparam * sizeof(float), st));
     const Conv& c = u->convs.back();
-    float* dW = u->grad + c.w_off;
-    float* db = u->grad + c.b_off;
-    // bias: db = sum_p dout[p][0]
-    RC(unet_bias_grad(st, dout, db, P, 1, 8));
-    // the output gradient is copied out before the weight-gradient transposes reuse the scratch
-    __nv_bfloat16* doutc = u->colt;
-    PAT_CUDA(cudaMemcpyAsync(doutc, dout, P * 8 * sizeof(__nv_bfloat16), cudaMemcpyDeviceToDevice, st));
-    // dW[0][ci] = sum_p dout[p] top[p][ci]: transposes [8][P] and [cin][P]
-    RC(unet_transpose(st, doutc, u->dt, int(P), 8, 8));
-    RC(unet_transpose(st, top.y, u->col, int(P), c.cin, c.cin));
-    PAT_CUDA(cudaMemsetAsync(dW, 0, c.nw() * sizeof(float), st));
-    {
-        const int splitk = std::max(1, std::min(64, int(P / 4096)));
-        // rows 1..7 of the transposed output gradient are zero; only row 0 (= dW) is kept
-        RC(net_gemm(u, st, u->dt, int(P), u->col, int(P), 1, c.cin, int(P), nullptr, 0, dW, c.cin, 2, splitk));
-    }
-    // data gradient of the final conv: dtop[p][ci] = dout[p] W[ci]: GEMM with K = 8 (W padded)
-    __nv_bfloat16* wpad = u->wt;
-    PAT_CUDA(cudaMemsetAsync(wpad, 0, size_t(c.cin) * 8 * sizeof(__nv_bfloat16), st));
-    RC(unet_copy_ch(st, u->wbf + c.wb_off, wpad, size_t(c.cin), 1, 1, 8, 0));
-    RC(net_gemm(u, st, doutc, 8, wpad, 8, int(P), c.cin, 8, nullptr, 0, top.g, c.cin, 0, 1));
-    // the rest of the network
+    RC(unet_head_bwd(st, u->out, d_target, top.y, u->wbf + c.wb_off, top.g, u->bpart, u->part, u->grad + c.w_off,
+                     u->grad + c.b_off, u->loss, P, c.cin));
+    // the rest of the network; every gradient below is already masked by its ReLU
     Layout L = layout_of(u);
     auto& A = u->acts;
     int ci = int(u->convs.size()) - 2;
@@ -404,31 +406,23 @@ static int loss_and_grads(pat_unet_s* u, cudaStream_t st, const float* d_in, con
         const Act& cat = A[L.dec_cat[d]];
         const Act& da = A[L.dec_a[d]];
         const Act& db2 = A[L.dec_b[d]];
-        const size_t Pl = size_t(B) * db2.H * db2.W;
-        RC(unet_relu_bwd(st, db2.g, db2.y, Pl * db2.C));
-        RC(conv_bwd(u, st, u->convs[ci--], da.y, da.C, B, db2.g, da.g));
-        RC(unet_relu_bwd(st, da.g, da.y, Pl * da.C));
-        RC(conv_bwd(u, st, u->convs[ci--], cat.y, cat.C, B, da.g, cat.g));
+        RC(conv_bwd(u, st, u->convs[ci--], da.y, da.C, B, db2.g, da.g, da.y));
+        RC(conv_bwd(u, st, u->convs[ci--], cat.y, cat.C, B, da.g, cat.g, nullptr));
         const Act& below = (d == 0) ? A[L.enc_b.back()] : A[L.dec_b[d - 1]];
-        RC(unet_upsample_bwd(st, cat.g, below.g, B, below.H, below.W, below.C, cat.C, 0));
+        RC(unet_upsample_bwd(st, cat.g, below.y, below.g, B, below.H, below.W, below.C, cat.C));
     }
     for (int l = u->levels - 1; l >= 0; --l) {
         const Act& ea = A[L.enc_a[l]];
         const Act& eb = A[L.enc_b[l]];
-        const size_t Pl = size_t(B) * eb.H * eb.W;
         if (l < u->levels - 1) {
-            const Act& pa = A[L.pool[l]];
-            RC(unet_maxpool_bwd(st, pa.g, u->pidx[l], eb.g, B, eb.H, eb.W, eb.C));
             const int d = u->levels - 2 - l;
             const Act& cat = A[L.dec_cat[d]];
             const int below_c = (d == 0) ? A[L.enc_b.back()].C : A[L.dec_b[d - 1]].C;
-            RC(unet_add_ch(st, eb.g, cat.g, Pl, eb.C, cat.C, below_c));
+            RC(unet_enc_bwd(st, A[L.pool[l]].g, u->pidx[l], cat.g, cat.C, below_c, eb.y, eb.g, B, eb.H, eb.W, eb.C));
         }
-        RC(unet_relu_bwd(st, eb.g, eb.y, Pl * eb.C));
-        RC(conv_bwd(u, st, u->convs[2 * l + 1], ea.y, ea.C, B, eb.g, ea.g));
-        RC(unet_relu_bwd(st, ea.g, ea.y, Pl * ea.C));
+        RC(conv_bwd(u, st, u->convs[2 * l + 1], ea.y, ea.C, B, eb.g, ea.g, ea.y));
         const Act& in = (l == 0) ? A[L.input] : A[L.pool[l - 1]];
-        RC(conv_bwd(u, st, u->convs[2 * l], in.y, in.C, B, ea.g, l == 0 ? nullptr : in.g));
+        RC(conv_bwd(u, st, u->convs[2 * l], in.y, in.C, B, ea.g, l == 0 ? nullptr : in.g, nullptr));
     }
     return PAT_OK;
 }
@@ -453,7 +447,7 @@ extern "C" int pat_unet_train_step(pat_unet u, const float* d_in, const float* d
     ++u->step;
     const float b1 = 0.9f, b2 = 0.999f;
     const float bc1 = 1.f - std::pow(b1, float(u->step)), bc2 = 1.f - std::pow(b2, float(u->step));
-    RC(unet_adam(st, u->param, nullptr, u->grad, u->m, u->v, u->nparam, lr, b1, b2, 1e-8f, bc1, bc2));
+    RC(unet_adam(st, u->param, u->grad, u->m, u->v, u->nparam, lr, b1, b2, 1e-8f, bc1, bc2));
     RC(sync_bf16(u, st));
     if (d_loss) PAT_CUDA(cudaMemcpyAsync(d_loss, u->loss, sizeof(double), cudaMemcpyDeviceToDevice, st));
     return PAT_OK;

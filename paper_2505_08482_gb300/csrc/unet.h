@@ -16,29 +16,45 @@ int unet_gemm(cudaStream_t st, const __nv_bfloat16* A, int lda, const __nv_bfloa
 bool unet_gemm_tc05_supported(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N, int K);
 int unet_gemm_tc05(cudaStream_t st, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N,
                    int K, const float* bias, int relu, void* C, int ldc, int out_mode, int splitk, int* d_status);
+// 3x3 convolution without im2col (unet_conv.cu): out[p][cout] (pitch ldo, bf16) = conv(in, W[cout][9][cin]) (+ bias)
+// (ReLU) (zero where mask <= 0, pitch cout); flip: taps reversed (data gradient)
+bool unet_conv_supported(const __nv_bfloat16* in, int ldin, int cin, int cout);
+int unet_conv(cudaStream_t st, const __nv_bfloat16* in, int ldin, const __nv_bfloat16* W, int B, int H, int Wd, int cin,
+              int cout, int flip, const float* bias, int relu, const __nv_bfloat16* mask, __nv_bfloat16* out, int ldo,
+              int* d_status);
+// dW[cout][kw] += sum_p dz[p][cout] in[p + off(tap)][c] at tap * cin + c < kw (taps 9, or 1 unshifted); dW zeroed by the caller
+bool unet_wgrad_supported(const __nv_bfloat16* in, int ldin, int cin, int cout);
+int unet_wgrad(cudaStream_t st, const __nv_bfloat16* in, int ldin, const __nv_bfloat16* dz, int B, int H, int Wd, int cin,
+               int taps, int cout, float* dW, int kw, int* d_status);
+
+struct ConvDesc {   // one convolution's weights in the parameter and bf16 arrays
+    int cin, cout, k;
+    size_t w_off, wb_off;
+};
+
 int unet_im2col(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* col, int B, int H, int W, int C, int ldc_in,
-                int flip);
+                int flip, int kp);
 int unet_transpose(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* out, int R, int C, int ld);
 int unet_maxpool(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* out, unsigned char* idx, int B, int H, int W,
                  int C);
-int unet_maxpool_bwd(cudaStream_t st, const __nv_bfloat16* dout, const unsigned char* idx, __nv_bfloat16* din, int B,
-                     int H, int W, int C);
-int unet_upsample(cudaStream_t st, const __nv_bfloat16* src, __nv_bfloat16* dst, int B, int Hs, int Ws, int C, int ldi,
-                  int ldo, int off);
-int unet_upsample_bwd(cudaStream_t st, const __nv_bfloat16* dst, __nv_bfloat16* dsrc, int B, int Hs, int Ws, int C,
-                      int ldo, int off);
-int unet_copy_ch(cudaStream_t st, const __nv_bfloat16* src, __nv_bfloat16* dst, size_t P, int C, int lds, int ldd,
-                 int off);
-int unet_add_ch(cudaStream_t st, __nv_bfloat16* dst, const __nv_bfloat16* src, size_t P, int C, int lds, int off);
+int unet_enc_bwd(cudaStream_t st, const __nv_bfloat16* dout, const unsigned char* idx, const __nv_bfloat16* cat, int ldcat,
+                 int off, const __nv_bfloat16* y, __nv_bfloat16* din, int B, int H, int W, int C);
+int unet_concat(cudaStream_t st, const __nv_bfloat16* src, const __nv_bfloat16* skip, __nv_bfloat16* cat, int B, int Hs,
+                int Ws, int Cs, int Ck);
+int unet_upsample_bwd(cudaStream_t st, const __nv_bfloat16* cat, const __nv_bfloat16* y, __nv_bfloat16* dsrc, int B, int Hs,
+                      int Ws, int C, int ldo);
 int unet_relu_bwd(cudaStream_t st, __nv_bfloat16* g, const __nv_bfloat16* y, size_t n);
-int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, size_t P, int C, int ld);
-int unet_mse(cudaStream_t st, const float* pred, const float* tgt, __nv_bfloat16* grad, size_t n, int ld,
-             double* part, double* loss);
-int unet_adam(cudaStream_t st, float* w, __nv_bfloat16* wb, const float* g, float* m, float* v, size_t n, float lr,
-              float b1, float b2, float eps, float bc1, float bc2);
-int unet_f32_to_bf16(cudaStream_t st, const float* a, __nv_bfloat16* b, size_t n);
-int unet_bf16_to_f32(cudaStream_t st, const __nv_bfloat16* a, float* b, size_t n, int lda);
+size_t unet_part_floats(int C);   // scratch of the two-step sums below
+int unet_part_blocks();
+int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* part, size_t P, int C);
+int unet_head(cudaStream_t st, const __nv_bfloat16* y, const __nv_bfloat16* w, const float* bias, float* out, size_t P,
+              int C);
+int unet_head_bwd(cudaStream_t st, const float* out, const float* tgt, const __nv_bfloat16* y, const __nv_bfloat16* w,
+                  __nv_bfloat16* dy, float* part, double* lpart, float* dw, float* db, double* loss, size_t P, int C);
+int unet_adam(cudaStream_t st, float* w, const float* g, float* m, float* v, size_t n, float lr, float b1, float b2,
+              float eps, float bc1, float bc2);
+int unet_weights(cudaStream_t st, const float* param, __nv_bfloat16* wb, __nv_bfloat16* wt, const ConvDesc* desc, int n,
+                 size_t most);
 int unet_pack_input(cudaStream_t st, const float* in, __nv_bfloat16* out, int B, int Cin, int H, int W, int Cp);
-int unet_weight_t(cudaStream_t st, const __nv_bfloat16* W, __nv_bfloat16* Wt, int Cout, int Cin);
 
 }  // namespace pat

@@ -185,24 +185,29 @@ static unsigned nblk(size_t n) {
 }
 #define GRID_STRIDE(i, n) for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < (n); i += size_t(gridDim.x) * blockDim.x)
 
-// col[b][y][x][tap][c] = in[b][y+dy][x+dx][c] (zero outside), tap = (dy+1)*3 + (dx+1); flip: tap -> 8 - tap
+// Eight channels (16 bytes) per thread in the kernels below: NHWC with channel counts in multiples of 8.
+union Bf8 {
+    uint4 u;
+    __nv_bfloat16 h[8];
+};
+
+// col[b][y][x][tap * C + c] = in[b][y+dy][x+dx][c] (zero outside), tap = (dy+1)*3 + (dx+1); flip: tap -> 8 - tap;
+// rows of kp >= 9 C elements, the rest zero
 __global__ void k_im2col(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ col, int B, int H, int W,
-                         int C, int ldc_in, int flip) {
-    const size_t total = size_t(B) * H * W * 9 * C;
+                         int C, int ldc_in, int flip, int kp) {
+    const int C8 = C / 8, K8 = kp / 8;
+    const size_t total = size_t(B) * H * W * K8;
     GRID_STRIDE(i, total) {
-        const int c = int(i % C);
-        size_t r = i / C;
-        int tap = int(r % 9);
-        r /= 9;
-        const int x = int(r % W);
-        r /= W;
-        const int y = int(r % H);
-        const int b = int(r / H);
+        const int k = int(i % K8);
+        const size_t p = i / K8;
+        const int tap = k / C8, c = k - tap * C8;
+        const int x = int(p % W), y = int((p / W) % H);
         const int t = flip ? 8 - tap : tap;
         const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-        __nv_bfloat16 v = __float2bfloat16(0.f);
-        if (yy >= 0 && yy < H && xx >= 0 && xx < W) v = in[((size_t(b) * H + yy) * W + xx) * ldc_in + c];
-        col[i] = v;
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (tap < 9 && yy >= 0 && yy < H && xx >= 0 && xx < W)
+            v = *reinterpret_cast<const uint4*>(in + (p + (yy - y) * (long long)W + (xx - x)) * ldc_in + c * 8);
+        *reinterpret_cast<uint4*>(col + p * kp + size_t(k) * 8) = v;
     }
 }
 
@@ -230,167 +235,262 @@ __global__ void k_transpose(const __nv_bfloat16* __restrict__ in, __nv_bfloat16*
 // 2x2 max pooling (NHWC); idx records the argmax (0..3) for the backward
 __global__ void k_maxpool(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out,
                           unsigned char* __restrict__ idx, int B, int H, int W, int C) {
-    const int Ho = H / 2, Wo = W / 2;
-    const size_t total = size_t(B) * Ho * Wo * C;
+    const int Ho = H / 2, Wo = W / 2, C8 = C / 8;
+    const size_t total = size_t(B) * Ho * Wo * C8;
     GRID_STRIDE(i, total) {
-        const int c = int(i % C);
-        size_t r = i / C;
+        const int c = int(i % C8) * 8;
+        size_t r = i / C8;
         const int x = int(r % Wo);
         r /= Wo;
         const int y = int(r % Ho);
         const int b = int(r / Ho);
-        float best = -3.0e38f;
-        int bi = 0;
-        for (int q = 0; q < 4; ++q) {
-            const float v = __bfloat162float(in[((size_t(b) * H + 2 * y + q / 2) * W + 2 * x + q % 2) * C + c]);
-            if (v > best) {
-                best = v;
-                bi = q;
-            }
-        }
-        out[i] = __float2bfloat16(best);
-        idx[i] = (unsigned char)bi;
-    }
-}
-
-__global__ void k_maxpool_bwd(const __nv_bfloat16* __restrict__ dout, const unsigned char* __restrict__ idx,
-                              __nv_bfloat16* __restrict__ din, int B, int H, int W, int C) {
-    const int Ho = H / 2, Wo = W / 2;
-    const size_t total = size_t(B) * Ho * Wo * C;
-    GRID_STRIDE(i, total) {
-        const int c = int(i % C);
-        size_t r = i / C;
-        const int x = int(r % Wo);
-        r /= Wo;
-        const int y = int(r % Ho);
-        const int b = int(r / Ho);
+        Bf8 v[4], o;
         for (int q = 0; q < 4; ++q)
-            din[((size_t(b) * H + 2 * y + q / 2) * W + 2 * x + q % 2) * C + c] =
-                q == idx[i] ? dout[i] : __float2bfloat16(0.f);
+            v[q].u = *reinterpret_cast<const uint4*>(in + ((size_t(b) * H + 2 * y + q / 2) * W + 2 * x + q % 2) * C + c);
+        unsigned char ix[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float best = -3.0e38f;
+            int bi = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float f = __bfloat162float(v[q].h[j]);
+                if (f > best) {
+                    best = f;
+                    bi = q;
+                }
+            }
+            o.h[j] = __float2bfloat16(best);
+            ix[j] = (unsigned char)bi;
+        }
+        *reinterpret_cast<uint4*>(out + i * 8) = o.u;
+        *reinterpret_cast<uint2*>(idx + i * 8) = *reinterpret_cast<const uint2*>(ix);
     }
 }
 
-// nearest 2x upsampling of src (C channels, pitch ldi) into dst channels [off, off+C) of pitch ldo
-__global__ void k_upsample(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst, int B, int Hs,
-                           int Ws, int C, int ldi, int ldo, int off) {
-    const int H = Hs * 2, W = Ws * 2;
-    const size_t total = size_t(B) * H * W * C;
+// gradient of an encoder output y (pooled and, from channel `off` of cat's gradient, skipped to the
+// decoder): din = [y > 0] (unpool(dout) + cat[off ..]), rounded as the two steps one after the other
+__global__ void k_enc_bwd(const __nv_bfloat16* __restrict__ dout, const unsigned char* __restrict__ idx,
+                          const __nv_bfloat16* __restrict__ cat, int ldcat, int off, const __nv_bfloat16* __restrict__ yv,
+                          __nv_bfloat16* __restrict__ din, int B, int H, int W, int C) {
+    const int Ho = H / 2, Wo = W / 2, C8 = C / 8;
+    const size_t total = size_t(B) * Ho * Wo * C8;
     GRID_STRIDE(i, total) {
-        const int c = int(i % C);
-        size_t r = i / C;
-        const int x = int(r % W);
-        r /= W;
-        const int y = int(r % H);
-        const int b = int(r / H);
-        dst[((size_t(b) * H + y) * W + x) * ldo + off + c] = src[((size_t(b) * Hs + y / 2) * Ws + x / 2) * ldi + c];
+        const int c = int(i % C8) * 8;
+        size_t r = i / C8;
+        const int x = int(r % Wo);
+        r /= Wo;
+        const int y = int(r % Ho);
+        const int b = int(r / Ho);
+        Bf8 d;
+        d.u = *reinterpret_cast<const uint4*>(dout + i * 8);
+        uint2 ixu = *reinterpret_cast<const uint2*>(idx + i * 8);
+        const unsigned char* ix = reinterpret_cast<const unsigned char*>(&ixu);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const size_t p = (size_t(b) * H + 2 * y + q / 2) * W + 2 * x + q % 2;
+            Bf8 s, yy, o;
+            s.u = *reinterpret_cast<const uint4*>(cat + p * ldcat + off + c);
+            yy.u = *reinterpret_cast<const uint4*>(yv + p * C + c);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float v = (ix[j] == q ? __bfloat162float(d.h[j]) : 0.f) + __bfloat162float(s.h[j]);
+                o.h[j] = __float2bfloat16(__bfloat162float(yy.h[j]) > 0.f ? v : 0.f);
+            }
+            *reinterpret_cast<uint4*>(din + p * C + c) = o.u;
+        }
     }
 }
 
-// backward of the nearest upsampling: sum of the 4 children (fp32 math)
-__global__ void k_upsample_bwd(const __nv_bfloat16* __restrict__ dst, __nv_bfloat16* __restrict__ dsrc, int B,
-                               int Hs, int Ws, int C, int ldo, int off) {
-    const int H = Hs * 2, W = Ws * 2;
-    const size_t total = size_t(B) * Hs * Ws * C;
+// decoder input: cat = [nearest 2x upsampling of src (Cs channels) | skip (Ck channels)]
+__global__ void k_concat(const __nv_bfloat16* __restrict__ src, const __nv_bfloat16* __restrict__ skip,
+                         __nv_bfloat16* __restrict__ cat, int B, int Hs, int Ws, int Cs, int Ck) {
+    const int H = Hs * 2, W = Ws * 2, C8 = (Cs + Ck) / 8;
+    const size_t total = size_t(B) * H * W * C8;
     GRID_STRIDE(i, total) {
-        const int c = int(i % C);
-        size_t r = i / C;
+        const int c = int(i % C8) * 8;
+        const size_t p = i / C8;
+        const int x = int(p % W), y = int((p / W) % H);
+        const int b = int(p / (size_t(W) * H));
+        const __nv_bfloat16* s = c < Cs ? src + ((size_t(b) * Hs + y / 2) * Ws + x / 2) * Cs + c : skip + p * Ck + (c - Cs);
+        *reinterpret_cast<uint4*>(cat + i * 8) = *reinterpret_cast<const uint4*>(s);
+    }
+}
+
+// backward of the nearest upsampling and of the ReLU below it: dsrc = [y > 0] sum of the 4 children of
+// the first C channels of cat's gradient (fp32 sum)
+__global__ void k_upsample_bwd(const __nv_bfloat16* __restrict__ cat, const __nv_bfloat16* __restrict__ yv,
+                               __nv_bfloat16* __restrict__ dsrc, int B, int Hs, int Ws, int C, int ldo) {
+    const int H = Hs * 2, W = Ws * 2, C8 = C / 8;
+    const size_t total = size_t(B) * Hs * Ws * C8;
+    GRID_STRIDE(i, total) {
+        const int c = int(i % C8) * 8;
+        size_t r = i / C8;
         const int x = int(r % Ws);
         r /= Ws;
         const int y = int(r % Hs);
         const int b = int(r / Hs);
-        float s = 0.f;
-        for (int q = 0; q < 4; ++q)
-            s += __bfloat162float(dst[((size_t(b) * H + 2 * y + q / 2) * W + 2 * x + q % 2) * ldo + off + c]);
-        dsrc[i] = __float2bfloat16(s);
-    }
-}
-
-// copy channels: dst[p][off + c] = src[p][c] (c < C), pitches lds / ldd; back: src <- dst slice
-__global__ void k_copy_ch(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst, size_t P, int C,
-                          int lds, int ldd, int off) {
-    GRID_STRIDE(i, P * C) {
-        const size_t p = i / C;
-        const int c = int(i % C);
-        dst[p * ldd + off + c] = src[p * lds + c];
-    }
-}
-
-// dst[p][c] += src[p][off + c]
-__global__ void k_add_ch(__nv_bfloat16* __restrict__ dst, const __nv_bfloat16* __restrict__ src, size_t P, int C,
-                         int lds, int off) {
-    GRID_STRIDE(i, P * C) {
-        const size_t p = i / C;
-        const int c = int(i % C);
-        dst[i] = __float2bfloat16(__bfloat162float(dst[i]) + __bfloat162float(src[p * lds + off + c]));
-    }
-}
-
-// weights for the data gradient: Wt[ci][tap][co] = W[co][tap][ci]
-__global__ void k_weight_t(const __nv_bfloat16* __restrict__ W, __nv_bfloat16* __restrict__ Wt, int Cout, int Cin) {
-    const size_t total = size_t(Cout) * 9 * Cin;
-    GRID_STRIDE(i, total) {
-        const int ci = int(i % Cin);
-        size_t r = i / Cin;
-        const int tap = int(r % 9);
-        const int co = int(r / 9);
-        Wt[(size_t(ci) * 9 + tap) * Cout + co] = W[i];
+        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            Bf8 v;
+            v.u = *reinterpret_cast<const uint4*>(cat + ((size_t(b) * H + 2 * y + q / 2) * W + 2 * x + q % 2) * ldo + c);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s[j] += __bfloat162float(v.h[j]);
+        }
+        Bf8 yy, o;
+        yy.u = *reinterpret_cast<const uint4*>(yv + i * 8);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) o.h[j] = __float2bfloat16(__bfloat162float(yy.h[j]) > 0.f ? s[j] : 0.f);
+        *reinterpret_cast<uint4*>(dsrc + i * 8) = o.u;
     }
 }
 
 // ReLU backward in place: g *= (y > 0)
-__global__ void k_relu_bwd(__nv_bfloat16* __restrict__ g, const __nv_bfloat16* __restrict__ y, size_t n) {
-    GRID_STRIDE(i, n) {
-        if (!(__bfloat162float(y[i]) > 0.f)) g[i] = __float2bfloat16(0.f);
+__global__ void k_relu_bwd(__nv_bfloat16* __restrict__ g, const __nv_bfloat16* __restrict__ y, size_t n8) {
+    GRID_STRIDE(i, n8) {
+        Bf8 a, b;
+        a.u = reinterpret_cast<const uint4*>(g)[i];
+        b.u = reinterpret_cast<const uint4*>(y)[i];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (!(__bfloat162float(b.h[j]) > 0.f)) a.h[j] = __float2bfloat16(0.f);
+        reinterpret_cast<uint4*>(g)[i] = a.u;
     }
 }
 
-// bias gradient: db[c] = sum_p g[p][c] (row pitch ld; one block per channel, fixed order)
-__global__ void k_bias_grad(const __nv_bfloat16* __restrict__ g, float* __restrict__ db, size_t P, int C, int ld) {
-    __shared__ float red[256];
-    for (int c = blockIdx.x; c < C; c += gridDim.x) {
-        float s = 0.f;
-        for (size_t p = threadIdx.x; p < P; p += blockDim.x) s += __bfloat162float(g[p * ld + c]);
-        red[threadIdx.x] = s;
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-            __syncthreads();
+// Bias gradient db[c] = sum_p g[p][c], in two steps of fixed order: block (b, z) sums the pixels b, b +
+// gridDim.x, ... (in groups of 256 / G) of 8 G channels from 64 z on into part[b][C]; then one block sums the parts.
+constexpr int kBiasBlocks = 296;
+__global__ void __launch_bounds__(256) k_bias_part(const __nv_bfloat16* __restrict__ g, float* __restrict__ part,
+                                                   size_t P, int C) {
+    __shared__ float red[256][9];
+    const int c0 = blockIdx.y * 64, G = min(8, (C - c0) / 8);
+    const int R = 256 / G, cg = threadIdx.x % G, pr = threadIdx.x / G;
+    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (pr < R)
+        for (size_t p = size_t(blockIdx.x) * R + pr; p < P; p += size_t(gridDim.x) * R) {
+            Bf8 v;
+            v.u = *reinterpret_cast<const uint4*>(g + p * C + c0 + cg * 8);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s[j] += __bfloat162float(v.h[j]);
         }
-        if (threadIdx.x == 0) db[c] = red[0];
-        __syncthreads();
-    }
-}
-
-// MSE loss L = mean (pred - target)^2 over n values; grad[i * ld] = 2 (pred - target) / n (bf16)
-__global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ tgt, __nv_bfloat16* __restrict__ grad,
-                      size_t n, int ld, double* __restrict__ loss_part) {
-    __shared__ double red[256];
-    double s = 0.0;
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x) {
-        const float d = pred[i] - tgt[i];
-        s += double(d) * d;
-        grad[i * ld] = __float2bfloat16(2.f * d / float(n));
-    }
-    red[threadIdx.x] = s;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = s[j];
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    if (threadIdx.x < 8 * G) {
+        const int c = threadIdx.x / 8, j = threadIdx.x % 8;
+        float t = 0.f;
+        for (int r = 0; r < R; ++r) t += red[r * G + c][j];
+        part[size_t(blockIdx.x) * C + c0 + c * 8 + j] = t;
+    }
+}
+__global__ void k_bias_sum(const float* __restrict__ part, int nblk, float* __restrict__ db, int C) {
+    const int c = blockIdx.x, lane = threadIdx.x;
+    float s = 0.f;
+    for (int b = lane; b < nblk; b += 32) s += part[size_t(b) * C + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) db[c] = s;
+}
+
+// Final 1x1 convolution to one channel: out[p] = sum_c y[p][c] w[c] + b.  A warp takes 16 pixels as the rows of
+// m16n8k16 MMAs whose second operand has w in column 0 and zeros elsewhere: the same 16-channel sums, in the
+// same order, as the GEMM above, for one read of y.
+__global__ void __launch_bounds__(256) k_head(const __nv_bfloat16* __restrict__ y, const __nv_bfloat16* __restrict__ w,
+                                              const float* __restrict__ bias, float* __restrict__ out, size_t P, int C) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t2 = (lane & 3) * 2;
+    const size_t warps = size_t(gridDim.x) * (blockDim.x >> 5);
+    for (size_t p0 = (size_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 16; p0 < P; p0 += warps * 16) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        auto pair = [&](const __nv_bfloat16* row, bool ok, int c) {
+            return ok && c < C ? *reinterpret_cast<const uint32_t*>(row + c) : 0u;
+        };
+        const bool ok0 = p0 + g < P, ok1 = p0 + g + 8 < P;
+        const __nv_bfloat16* r0 = y + (p0 + g) * C;
+        const __nv_bfloat16* r1 = r0 + size_t(8) * C;
+        for (int c = 0; c < C; c += 16) {
+            const uint32_t a[4] = {pair(r0, ok0, c + t2), pair(r1, ok1, c + t2), pair(r0, ok0, c + t2 + 8),
+                                   pair(r1, ok1, c + t2 + 8)};
+            gemm::mma_bf16(acc, a, pair(w, g == 0, c + t2), pair(w, g == 0, c + t2 + 8));
+        }
+        if (t2 == 0) {   // column 0 of rows g, g + 8
+            if (ok0) out[p0 + g] = acc[0] + bias[0];
+            if (ok1) out[p0 + g + 8] = acc[2] + bias[0];
+        }
+    }
+}
+
+// Loss L = mean (out - target)^2 and the backward of the final convolution in one pass over its input
+// y: d = bf16(2 (out - target) / n) per pixel, dy = [y > 0] bf16(d w), and per block the partial sums of
+// dW[c] = sum d y[c], db = sum d (part[b][C + 1]) and of the loss (lpart[b]).  Eight channels per thread.
+constexpr int kHeadBlocks = 296;
+__global__ void __launch_bounds__(256) k_head_bwd(const float* __restrict__ out, const float* __restrict__ tgt,
+                                                  const __nv_bfloat16* __restrict__ y,
+                                                  const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ dy,
+                                                  float* __restrict__ part, double* __restrict__ lpart, size_t P, int C) {
+    __shared__ float red[256][9];
+    __shared__ double lred[256];
+    const int G = C / 8, R = 256 / G;   // C <= 2048
+    const int cg = threadIdx.x % G, pr = threadIdx.x / G;
+    float wv[8], s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sb = 0.f;
+    double ls = 0.0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) wv[j] = __bfloat162float(w[cg * 8 + j]);
+    if (pr < R)
+        for (size_t p = size_t(blockIdx.x) * R + pr; p < P; p += size_t(gridDim.x) * R) {
+            const float e = out[p] - tgt[p];
+            const float d = __bfloat162float(__float2bfloat16(2.f * e / float(P)));
+            if (cg == 0) {
+                ls += double(e) * e;
+                sb += d;
+            }
+            Bf8 v, o;
+            v.u = *reinterpret_cast<const uint4*>(y + p * C + cg * 8);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float f = __bfloat162float(v.h[j]);
+                s[j] += d * f;
+                o.h[j] = __float2bfloat16(f > 0.f ? d * wv[j] : 0.f);
+            }
+            *reinterpret_cast<uint4*>(dy + p * C + cg * 8) = o.u;
+        }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = s[j];
+    red[threadIdx.x][8] = sb;
+    lred[threadIdx.x] = ls;
+    __syncthreads();
+    for (int t = threadIdx.x; t <= C; t += 256) {
+        float v = 0.f;
+        if (t < C)
+            for (int r = 0; r < R; ++r) v += red[r * G + t / 8][t % 8];
+        else
+            for (int r = 0; r < R; ++r) v += red[r * G][8];
+        part[size_t(blockIdx.x) * (C + 1) + t] = v;
+    }
+    for (int k = 128; k > 0; k >>= 1) {
         __syncthreads();
+        if (threadIdx.x < k) lred[threadIdx.x] += lred[threadIdx.x + k];
     }
-    if (threadIdx.x == 0) loss_part[blockIdx.x] = red[0];
+    if (threadIdx.x == 0) lpart[blockIdx.x] = lred[0];
 }
-
-__global__ void k_sum_d(const double* __restrict__ part, int n, double* __restrict__ out, double scale) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+__global__ void k_head_sum(const float* __restrict__ part, const double* __restrict__ lpart, int nblk,
+                           float* __restrict__ dw, float* __restrict__ db, double* __restrict__ loss, double scale, int C) {
+    const int lane = threadIdx.x, t = blockIdx.x;
+    if (t <= C) {
+        float s = 0.f;
+        for (int b = lane; b < nblk; b += 32) s += part[size_t(b) * (C + 1) + t];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) *(t < C ? dw + t : db) = s;
+    } else {
         double s = 0.0;
-        for (int i = 0; i < n; ++i) s += part[i];
-        *out = s * scale;
+        for (int b = lane; b < nblk; b += 32) s += lpart[b];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) *loss = s * scale;
     }
 }
 
-// Adam on fp32 master weights, refreshing the bf16 copies
-__global__ void k_adam(float* __restrict__ w, __nv_bfloat16* __restrict__ wb, const float* __restrict__ g,
-                       float* __restrict__ m, float* __restrict__ v, size_t n, float lr, float b1, float b2, float eps,
+// Adam on fp32 master weights
+__global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v, size_t n, float lr, float b1, float b2, float eps,
                        float bc1, float bc2) {
     GRID_STRIDE(i, n) {
         const float gi = g[i];
@@ -400,30 +500,43 @@ __global__ void k_adam(float* __restrict__ w, __nv_bfloat16* __restrict__ wb, co
         v[i] = vi;
         const float wi = w[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
         w[i] = wi;
-        if (wb) wb[i] = __float2bfloat16(wi);
     }
 }
 
-__global__ void k_f32_to_bf16(const float* __restrict__ a, __nv_bfloat16* __restrict__ b, size_t n) {
-    GRID_STRIDE(i, n) b[i] = __float2bfloat16(a[i]);
-}
-
-__global__ void k_bf16_to_f32(const __nv_bfloat16* __restrict__ a, float* __restrict__ b, size_t n, int lda) {
-    GRID_STRIDE(i, n) b[i] = __bfloat162float(a[i * lda]);
+// bf16 copies of every convolution's weights W[co][tap][ci] and, for the data gradient of the 3x3
+// ones, Wt[ci][tap][co]; blockIdx.y: convolution
+__global__ void k_weights(const float* __restrict__ param, __nv_bfloat16* __restrict__ wb, __nv_bfloat16* __restrict__ wt,
+                          const ConvDesc* __restrict__ desc) {
+    const ConvDesc d = desc[blockIdx.y];
+    const int taps = d.k * d.k;
+    const size_t n = size_t(d.cout) * taps * d.cin;
+    GRID_STRIDE(i, n) {
+        const __nv_bfloat16 v = __float2bfloat16(param[d.w_off + i]);
+        wb[d.wb_off + i] = v;
+        if (d.k == 3) {
+            const int ci = int(i % d.cin);
+            const size_t r = i / d.cin;
+            const int tap = int(r % 9), co = int(r / 9);
+            wt[d.wb_off + (size_t(ci) * 9 + tap) * d.cout + co] = v;
+        }
+    }
 }
 
 // input staging: fp32 [B][Cin][H][W] (NCHW, as the solver produces images) -> bf16 NHWC with C padded
-__global__ void k_pack_input(const float* __restrict__ in, __nv_bfloat16* __restrict__ out, int B, int Cin, int H,
-                             int W, int Cp) {
-    const size_t total = size_t(B) * H * W * Cp;
-    GRID_STRIDE(i, total) {
-        const int c = int(i % Cp);
-        size_t r = i / Cp;
-        const int x = int(r % W);
-        r /= W;
-        const int y = int(r % H);
-        const int b = int(r / H);
-        out[i] = c < Cin ? __float2bfloat16(in[((size_t(b) * Cin + c) * H + y) * W + x]) : __float2bfloat16(0.f);
+__global__ void k_pack_input(const float* __restrict__ in, __nv_bfloat16* __restrict__ out, int B, int Cin, size_t HW,
+                             int Cp) {
+    const int C8 = Cp / 8;
+    GRID_STRIDE(i, size_t(B) * HW * C8) {
+        const size_t p = i % HW;   // pixels fastest: the reads of a channel plane are contiguous
+        const int g = int((i / HW) % C8);
+        const int b = int(i / (HW * C8));
+        Bf8 v;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int c = g * 8 + j;
+            v.h[j] = __float2bfloat16(c < Cin ? in[(size_t(b) * Cin + c) * HW + p] : 0.f);
+        }
+        *reinterpret_cast<uint4*>(out + (size_t(b) * HW + p) * Cp + g * 8) = v.u;
     }
 }
 
@@ -436,8 +549,8 @@ __global__ void k_pack_input(const float* __restrict__ in, __nv_bfloat16* __rest
     } while (0)
 
 int unet_im2col(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* col, int B, int H, int W, int C, int ldc_in,
-                int flip) {
-    k_im2col<<<nblk(size_t(B) * H * W * 9 * C), 256, 0, st>>>(in, col, B, H, W, C, ldc_in, flip);
+                int flip, int kp) {
+    k_im2col<<<nblk(size_t(B) * H * W * (kp / 8)), 256, 0, st>>>(in, col, B, H, W, C, ldc_in, flip, kp);
     LAUNCH_CHECK("k_im2col");
     return PAT_OK;
 }
@@ -449,80 +562,71 @@ int unet_transpose(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* out,
 }
 int unet_maxpool(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* out, unsigned char* idx, int B, int H, int W,
                  int C) {
-    k_maxpool<<<nblk(size_t(B) * H * W * C / 4), 256, 0, st>>>(in, out, idx, B, H, W, C);
+    k_maxpool<<<nblk(size_t(B) * H * W * C / 32), 256, 0, st>>>(in, out, idx, B, H, W, C);
     LAUNCH_CHECK("k_maxpool");
     return PAT_OK;
 }
-int unet_maxpool_bwd(cudaStream_t st, const __nv_bfloat16* dout, const unsigned char* idx, __nv_bfloat16* din, int B,
-                     int H, int W, int C) {
-    k_maxpool_bwd<<<nblk(size_t(B) * H * W * C / 4), 256, 0, st>>>(dout, idx, din, B, H, W, C);
-    LAUNCH_CHECK("k_maxpool_bwd");
+int unet_enc_bwd(cudaStream_t st, const __nv_bfloat16* dout, const unsigned char* idx, const __nv_bfloat16* cat, int ldcat,
+                 int off, const __nv_bfloat16* y, __nv_bfloat16* din, int B, int H, int W, int C) {
+    k_enc_bwd<<<nblk(size_t(B) * H * W * C / 32), 256, 0, st>>>(dout, idx, cat, ldcat, off, y, din, B, H, W, C);
+    LAUNCH_CHECK("k_enc_bwd");
     return PAT_OK;
 }
-int unet_upsample(cudaStream_t st, const __nv_bfloat16* src, __nv_bfloat16* dst, int B, int Hs, int Ws, int C, int ldi,
-                  int ldo, int off) {
-    k_upsample<<<nblk(size_t(B) * Hs * Ws * 4 * C), 256, 0, st>>>(src, dst, B, Hs, Ws, C, ldi, ldo, off);
-    LAUNCH_CHECK("k_upsample");
+int unet_concat(cudaStream_t st, const __nv_bfloat16* src, const __nv_bfloat16* skip, __nv_bfloat16* cat, int B, int Hs,
+                int Ws, int Cs, int Ck) {
+    k_concat<<<nblk(size_t(B) * Hs * Ws * 4 * (Cs + Ck) / 8), 256, 0, st>>>(src, skip, cat, B, Hs, Ws, Cs, Ck);
+    LAUNCH_CHECK("k_concat");
     return PAT_OK;
 }
-int unet_upsample_bwd(cudaStream_t st, const __nv_bfloat16* dst, __nv_bfloat16* dsrc, int B, int Hs, int Ws, int C,
-                      int ldo, int off) {
-    k_upsample_bwd<<<nblk(size_t(B) * Hs * Ws * C), 256, 0, st>>>(dst, dsrc, B, Hs, Ws, C, ldo, off);
+int unet_upsample_bwd(cudaStream_t st, const __nv_bfloat16* cat, const __nv_bfloat16* y, __nv_bfloat16* dsrc, int B, int Hs,
+                      int Ws, int C, int ldo) {
+    k_upsample_bwd<<<nblk(size_t(B) * Hs * Ws * C / 8), 256, 0, st>>>(cat, y, dsrc, B, Hs, Ws, C, ldo);
     LAUNCH_CHECK("k_upsample_bwd");
     return PAT_OK;
 }
-int unet_copy_ch(cudaStream_t st, const __nv_bfloat16* src, __nv_bfloat16* dst, size_t P, int C, int lds, int ldd,
-                 int off) {
-    k_copy_ch<<<nblk(P * C), 256, 0, st>>>(src, dst, P, C, lds, ldd, off);
-    LAUNCH_CHECK("k_copy_ch");
-    return PAT_OK;
-}
-int unet_add_ch(cudaStream_t st, __nv_bfloat16* dst, const __nv_bfloat16* src, size_t P, int C, int lds, int off) {
-    k_add_ch<<<nblk(P * C), 256, 0, st>>>(dst, src, P, C, lds, off);
-    LAUNCH_CHECK("k_add_ch");
-    return PAT_OK;
-}
-int unet_weight_t(cudaStream_t st, const __nv_bfloat16* W, __nv_bfloat16* Wt, int Cout, int Cin) {
-    k_weight_t<<<nblk(size_t(Cout) * 9 * Cin), 256, 0, st>>>(W, Wt, Cout, Cin);
-    LAUNCH_CHECK("k_weight_t");
-    return PAT_OK;
-}
 int unet_relu_bwd(cudaStream_t st, __nv_bfloat16* g, const __nv_bfloat16* y, size_t n) {
-    k_relu_bwd<<<nblk(n), 256, 0, st>>>(g, y, n);
+    k_relu_bwd<<<nblk(n / 8), 256, 0, st>>>(g, y, n / 8);
     LAUNCH_CHECK("k_relu_bwd");
     return PAT_OK;
 }
-int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, size_t P, int C, int ld) {
-    k_bias_grad<<<std::min(C, 1024), 256, 0, st>>>(g, db, P, C, ld);
-    LAUNCH_CHECK("k_bias_grad");
+int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* part, size_t P, int C) {
+    const unsigned nb = unsigned(std::min<size_t>(kBiasBlocks, (P + 31) / 32));
+    k_bias_part<<<dim3(nb, (C + 63) / 64), 256, 0, st>>>(g, part, P, C);
+    LAUNCH_CHECK("k_bias_part");
+    k_bias_sum<<<C, 32, 0, st>>>(part, int(nb), db, C);
+    LAUNCH_CHECK("k_bias_sum");
     return PAT_OK;
 }
-int unet_mse(cudaStream_t st, const float* pred, const float* tgt, __nv_bfloat16* grad, size_t n, int ld,
-             double* part, double* loss) {
-    k_mse<<<256, 256, 0, st>>>(pred, tgt, grad, n, ld, part);
-    LAUNCH_CHECK("k_mse");
-    k_sum_d<<<1, 32, 0, st>>>(part, 256, loss, 1.0 / double(n));
-    LAUNCH_CHECK("k_sum_d");
+size_t unet_part_floats(int C) { return size_t(kBiasBlocks > kHeadBlocks ? kBiasBlocks : kHeadBlocks) * (C + 1); }
+int unet_part_blocks() { return kHeadBlocks; }
+int unet_head(cudaStream_t st, const __nv_bfloat16* y, const __nv_bfloat16* w, const float* bias, float* out, size_t P,
+              int C) {
+    k_head<<<unsigned(std::min<size_t>((P + 127) / 128, 65535)), 256, 0, st>>>(y, w, bias, out, P, C);
+    LAUNCH_CHECK("k_head");
     return PAT_OK;
 }
-int unet_adam(cudaStream_t st, float* w, __nv_bfloat16* wb, const float* g, float* m, float* v, size_t n, float lr,
-              float b1, float b2, float eps, float bc1, float bc2) {
-    k_adam<<<nblk(n), 256, 0, st>>>(w, wb, g, m, v, n, lr, b1, b2, eps, bc1, bc2);
+int unet_head_bwd(cudaStream_t st, const float* out, const float* tgt, const __nv_bfloat16* y, const __nv_bfloat16* w,
+                  __nv_bfloat16* dy, float* part, double* lpart, float* dw, float* db, double* loss, size_t P, int C) {
+    k_head_bwd<<<kHeadBlocks, 256, 0, st>>>(out, tgt, y, w, dy, part, lpart, P, C);
+    LAUNCH_CHECK("k_head_bwd");
+    k_head_sum<<<C + 2, 32, 0, st>>>(part, lpart, kHeadBlocks, dw, db, loss, 1.0 / double(P), C);
+    LAUNCH_CHECK("k_head_sum");
+    return PAT_OK;
+}
+int unet_adam(cudaStream_t st, float* w, const float* g, float* m, float* v, size_t n, float lr, float b1, float b2,
+              float eps, float bc1, float bc2) {
+    k_adam<<<nblk(n), 256, 0, st>>>(w, g, m, v, n, lr, b1, b2, eps, bc1, bc2);
     LAUNCH_CHECK("k_adam");
     return PAT_OK;
 }
-int unet_f32_to_bf16(cudaStream_t st, const float* a, __nv_bfloat16* b, size_t n) {
-    k_f32_to_bf16<<<nblk(n), 256, 0, st>>>(a, b, n);
-    LAUNCH_CHECK("k_f32_to_bf16");
-    return PAT_OK;
-}
-int unet_bf16_to_f32(cudaStream_t st, const __nv_bfloat16* a, float* b, size_t n, int lda) {
-    k_bf16_to_f32<<<nblk(n), 256, 0, st>>>(a, b, n, lda);
-    LAUNCH_CHECK("k_bf16_to_f32");
+int unet_weights(cudaStream_t st, const float* param, __nv_bfloat16* wb, __nv_bfloat16* wt, const ConvDesc* desc, int n,
+                 size_t most) {
+    k_weights<<<dim3(std::min(nblk(most), 1024u), n), 256, 0, st>>>(param, wb, wt, desc);
+    LAUNCH_CHECK("k_weights");
     return PAT_OK;
 }
 int unet_pack_input(cudaStream_t st, const float* in, __nv_bfloat16* out, int B, int Cin, int H, int W, int Cp) {
-    k_pack_input<<<nblk(size_t(B) * H * W * Cp), 256, 0, st>>>(in, out, B, Cin, H, W, Cp);
+    k_pack_input<<<nblk(size_t(B) * H * W * Cp / 8), 256, 0, st>>>(in, out, B, Cin, size_t(H) * W, Cp);
     LAUNCH_CHECK("k_pack_input");
     return PAT_OK;
 }

@@ -28,6 +28,7 @@
 
 #include "pat_internal.h"
 #include "sync.cuh"
+#include "tc05.cuh"
 #include "unet.h"
 
 namespace pat {
@@ -35,7 +36,6 @@ namespace tc05 {
 
 constexpr int BM = 128, BK = 64, STAGES = 4, THREADS = 128;
 constexpr uint32_t TILE_A = BM * BK * 2;            // bytes of one A tile (128 rows x 64 K-elements)
-constexpr uint64_t kWaitNs = 200000000ull;          // 0.2 s per wait
 constexpr int GROUP_M = 8;                          // tile rows per group of the tile order
 
 // Shared memory of a CTA with an N tile of BN: the 4-stage ring of A and B tiles (1024-byte
@@ -53,40 +53,6 @@ __host__ __device__ constexpr uint32_t idesc() {
     return (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) | (uint32_t(BM >> 4) << 24);
 }
 
-// Shared-memory matrix descriptor of a K-major tile with the 128-byte swizzle: start
-// address / 16 (bits 0-13), leading byte offset / 16 (bits 16-29; not used by swizzled
-// K-major tiles), stride byte offset / 16 = 1024 / 16 (bits 32-45: 8 rows of 128 bytes),
-// descriptor version 1 (bits 46-47), swizzle mode 2 = 128 bytes (bits 61-63).
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    return uint64_t((saddr & 0x3FFFFu) >> 4) | (uint64_t(1) << 16) | (uint64_t(1024 >> 4) << 32) |
-           (uint64_t(1) << 46) | (uint64_t(2) << 61);
-}
-
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* mb) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            s_addr(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(s_addr(mb))
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t id, uint32_t acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(da), "l"(db), "r"(id), "r"(acc)
-        : "memory");
-}
-
-// arrive on mb once every MMA issued so far by this thread has completed
-__device__ __forceinline__ void mma_commit(uint64_t* mb) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_addr(mb))
-                 : "memory");
-}
-
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
 struct Args {
     int M, N, K;
     int ksplit;            // K range per blockIdx.z (a multiple of BK)
@@ -95,6 +61,7 @@ struct Args {
     void* C;
     int ldc;
     int out_mode;          // 0 bf16 store, 1 fp32 store, 2 fp32 atomic add
+    int vec;               // rows of C allow 16-byte stores
     int* status;           // device status word (bit PAT_STATUS_TC05 on a given-up wait), or null
 };
 
@@ -194,7 +161,28 @@ __global__ void __launch_bounds__(THREADS, 1) k_gemm_tc05(const __grid_constant_
                   "=r"(v[15])
                 : "r"(taddr + uint32_t(c0)));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < a.M) {
+            const size_t orow = size_t(row) * a.ldc + n0 + c0;
+            if (row < a.M && a.vec && a.out_mode < 2 && n0 + c0 + 16 <= a.N) {   // 16-byte stores
+                float f[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    f[j] = __uint_as_float(v[j]);
+                    if (a.bias) f[j] += a.bias[n0 + c0 + j];
+                    if (a.relu) f[j] = fmaxf(f[j], 0.f);
+                }
+                if (a.out_mode == 0) {
+                    __nv_bfloat162 w[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) w[j] = __floats2bfloat162_rn(f[2 * j], f[2 * j + 1]);
+                    uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(a.C) + orow);
+                    o[0] = reinterpret_cast<const uint4*>(w)[0];
+                    o[1] = reinterpret_cast<const uint4*>(w)[1];
+                } else {
+                    float4* o = reinterpret_cast<float4*>(static_cast<float*>(a.C) + orow);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[j] = make_float4(f[4 * j], f[4 * j + 1], f[4 * j + 2], f[4 * j + 3]);
+                }
+            } else if (row < a.M) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const int n = n0 + c0 + j;
@@ -308,7 +296,8 @@ int unet_gemm_tc05(cudaStream_t st, const __nv_bfloat16* A, int lda, const __nv_
     splitk = std::max(1, splitk);
     int ks = (K + splitk - 1) / splitk;
     ks = (ks + tc05::BK - 1) / tc05::BK * tc05::BK;   // split boundaries on whole K boxes
-    tc05::Args a{M, N, K, ks, bias, relu, C, ldc, out_mode, d_status};
+    const int vec = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && ldc % 8 == 0;
+    tc05::Args a{M, N, K, ks, bias, relu, C, ldc, out_mode, vec, d_status};
     // the wider N tile halves the A traffic per MMA, where N allows it and the product still has
     // at least two waves of tiles (fewer tiles would leave SMs idle)
     int dev = 0, sms = 148;
