@@ -127,7 +127,7 @@ int run_adj(const Launch& L, const Ws& w, const float* r, int n_hi, int n_lo, bo
             float sg, float sd) {
     if (L.split) return split_adjoint(L, w, r, n_hi, n_lo, first, h, hbase);
     for (int n = n_hi; n >= n_lo; --n) {
-        RC(launch_row_adj_rho(L, w, (first && n == n_hi) ? 1 : 0, r, n, h, n - hbase));
+        RC(launch_row_adj_rho(L, w, (first && n == n_hi) ? 1 : 0, r, n, h, n - hbase, n == n_hi));
         RC(launch_col(L, w.A2, w.B2, 1, 0, sg));
         RC(launch_row_adj_u(L, w));
         RC(launch_col(L, w.A2, w.B2, 2, 1, sd));

@@ -732,12 +732,12 @@ int launch_col(const Launch& L, float2* A, float2* B, int mode, int op, float sc
 }
 
 int launch_row_adj_rho(const Launch& L, const Ws& w, int first, const float* resid, int tstep, const float* hist,
-                       int hist_slot) {
+                       int hist_slot, bool opens_segment) {
     const pat_plan_s* p = L.p;
     prof_begin(PAT_K_ROW_ADJ_RHO, L.st);
     if (p->fast)
         p->fast->row_adj_rho(geo_ws(p, w), L.st, w.A2, w.B2, w.rbx, w.rby, w.cbar, w.cg, first, resid, tstep, hist,
-                             hist_slot);
+                             hist_slot, !opens_segment);
     else
         k_row_adj_rho<<<row_grid(p), 256, p->smem_row, L.st>>>(geo(p), w.A2, w.B2, w.rbx, w.rby, w.cbar, w.cg,
                                                                first, resid, tstep, hist, hist_slot, p->R);

@@ -52,7 +52,7 @@ struct FixedOps {
     void (*row_rho)(const Geo&, cudaStream_t, float2*, const float2*, float*, float*, const float*, int mode,
                     const float* p0, float* y, int tstep, float* hist, int hist_slot);
     void (*row_adj_rho)(const Geo&, cudaStream_t, float2*, float2*, float*, float*, float*, const float*,
-                        int first, const float* resid, int tstep, const float* hist, int hist_slot);
+                        int first, const float* resid, int tstep, const float* hist, int hist_slot, bool pdl);
     // column pass for passes that run alone on the GPU (nullptr: col)
     void (*col_solo)(const Geo&, cudaStream_t, float2*, float2*, int mode, int op, float scale);
     // row passes of the segment recompute, which shares the GPU with the adjoint (nullptr: row_u, row_rho)
@@ -833,8 +833,10 @@ __global__ void __launch_bounds__(RR * Fft2<N1, N2>::T) kf_row_adj_rho(Geo g, fl
             s_ewb[e - e0] = sw.y * v;
         }
     // The pressure history is written by the segment recompute on the other stream, which this
-    // segment's first kernel waits for through an event (a full dependency), or by the forward
-    // sweep: never by the kernel just before, so it is fetched before the wait as well.
+    // segment's first kernel waits for through an event, or by the forward sweep: never by the
+    // kernel just before, so it is fetched before the wait as well.  That first kernel is an ordinary
+    // launch: with the programmatic attribute a captured graph makes its edge from the recompute
+    // programmatic too, and it would read the history before the recompute has finished.
     const int hslot = in_range_or_zero(hist_slot, g.s_eff, g.status);
     const float* hr = hist + (size_t(k) * g.s_eff + hslot) * N * N + size_t(yy) * N;
     if constexpr (STAGE) {
@@ -994,9 +996,9 @@ struct FixedImpl {
     }
     static void row_adj_rho(const Geo& g, cudaStream_t st, float2* A2, float2* B2, float* rbx, float* rby,
                             float* cbar, const float* cg, int first, const float* resid, int tstep,
-                            const float* hist, int slot) {
+                            const float* hist, int slot, bool pdl) {
         dim3 grid((F::N + RR - 1) / RR, g.K);
-        launch_pdl(kf_row_adj_rho<N1, N2, RR, STAGE>, grid, dim3(RR * F::T), smem_adj, st, true, g, A2, B2, rbx,
+        launch_pdl(kf_row_adj_rho<N1, N2, RR, STAGE>, grid, dim3(RR * F::T), smem_adj, st, pdl, g, A2, B2, rbx,
                    rby, cbar, cg, first, resid, tstep, hist, slot);
     }
     static FixedOps ops() {

@@ -173,8 +173,9 @@ int launch_forward_persistent(const Launch& L, const Ws& w, const float* p0, flo
 // op 0: G multipliers, op 1: D multipliers
 int launch_col(const Launch& L, float2* A, float2* B, int mode, int op, float scale);
 // adjoint
-int launch_row_adj_rho(const Launch& L, const Ws& w, int first, const float* resid, int tstep,
-                       const float* hist, int hist_slot);
+// opens_segment: the segment's first adjoint step, which waits for the recompute of the pressure history
+int launch_row_adj_rho(const Launch& L, const Ws& w, int first, const float* resid, int tstep, const float* hist,
+                       int hist_slot, bool opens_segment);
 int launch_row_adj_u(const Launch& L, const Ws& w);
 int launch_row_adj_final1(const Launch& L, const Ws& w, int first, const float* resid, float* grad_p0);
 int launch_row_adj_final2(const Launch& L, const Ws& w, const float* p0, float* grad_p0);
