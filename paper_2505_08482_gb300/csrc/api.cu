@@ -11,12 +11,21 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "pat_internal.h"
 #include "vec.h"
 
 using namespace pat;
+
+float pat::scale_g(const pat_plan_s* p) {
+    return float(p->g.dt / p->g.rho0 / (double(p->ng) * p->ng) * std::pow(1.0 + p->gain, -2.0));
+}
+float pat::scale_d(const pat_plan_s* p) {
+    const double n2 = double(p->ng) * p->ng, target = p->g.dt / n2 * (p->g.dt / n2) * std::pow(1.0 + p->gain, -4.0);
+    return float(target / double(scale_g(p)));
+}
 
 namespace {
 
@@ -25,13 +34,6 @@ namespace {
         int rc_ = (x);          \
         if (rc_ != PAT_OK) return rc_; \
     } while (0)
-
-float scale_g(const pat_plan_s* p) {  // dt/rho0 G, inverse 2-D FFT normalisation folded in
-    return float(p->g.dt / p->g.rho0 / (double(p->ng) * p->ng));
-}
-float scale_d(const pat_plan_s* p) {  // dt rho0 D
-    return float(p->g.dt * p->g.rho0 / (double(p->ng) * p->ng));
-}
 
 // one forward step n -> n+1 given the row spectrum of p^n in A
 int step(const Launch& L, const Ws& w, int n, float* y, float* hist, int hist_slot) {
@@ -151,8 +153,7 @@ int reverse_sweep(pat_plan_s* p, const float* p0, const float* r, float* grad_p0
         PAT_CUDA(cudaMemsetAsync(w.ubx, 0, 4 * f * sizeof(float), st));
     }
     PAT_CUDA(cudaMemsetAsync(w.cbar, 0, size_t(p->K) * p->n * p->n * sizeof(float), st));
-    const float sg = float(p->g.dt * p->g.rho0 / (double(p->ng) * p->ng));   // dt rho0 G t
-    const float sd = float(p->g.dt / p->g.rho0 / (double(p->ng) * p->ng));   // dt/rho0 D t'
+    const float sg = scale_d(p), sd = scale_g(p);   // dt rho0 G t, dt/rho0 D t'
     cudaStream_t R = p->side;
     const int last = p->nseg - 1;
     // the side stream starts after everything issued so far on st (forward sweep, residual)

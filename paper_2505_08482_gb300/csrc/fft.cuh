@@ -42,6 +42,14 @@ __host__ __device__ __forceinline__ float2 cscale(float2 a, float s) {
     return make_float2(a.x * s, a.y * s);
 #endif
 }
+// part by part
+__host__ __device__ __forceinline__ float2 cprod(float2 a, float2 b) {
+#ifdef __CUDA_ARCH__
+    return __fmul2_rn(a, b);
+#else
+    return make_float2(a.x * b.x, a.y * b.y);
+#endif
+}
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }

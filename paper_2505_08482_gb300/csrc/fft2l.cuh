@@ -188,6 +188,30 @@ struct Fft2 {
             Z[(k1 * P2 + n2) * S] = v;
         });
     }
+    // The same transforms with all twiddles on the A side, in registers: w[k1] = W_N^{n2 k1} of the thread's n2,
+    // loaded once and used by every forward and inverse transform of the sequence.  Same values, same results.
+    template <int S = 1>
+    __host__ __device__ static __forceinline__ void fwd_a_w(float2 (&a)[N1], int n2, float2* Z, const float2 (&w)[N1]) {
+        dft<N1, false>(a);
+        static_for<0, N1>([&](auto kI) {
+            constexpr int k1 = decltype(kI)::value;
+            Z[(k1 * P2 + n2) * S] = k1 > 0 ? cmul(a[k1], w[k1]) : a[k1];
+        });
+    }
+    template <int S = 1>
+    __host__ __device__ static __forceinline__ void inv_b_w(float2 (&b)[N2], int k1, float2* Z) {
+        dft<N2, true>(b);
+        static_for<0, N2>([&](auto nI) { Z[(k1 * P2 + decltype(nI)::value) * S] = b[decltype(nI)::value]; });
+    }
+    template <int S = 1>
+    __host__ __device__ static __forceinline__ void inv_a_load_w(float2 (&a)[N1], int n2, const float2* Z,
+                                                                 const float2 (&w)[N1]) {
+        static_for<0, N1>([&](auto kI) {
+            constexpr int k1 = decltype(kI)::value;
+            const float2 v = Z[(k1 * P2 + n2) * S];
+            a[k1] = k1 > 0 ? cmulc(v, w[k1]) : v;
+        });
+    }
     // twA and twB (N entries each) from the natural-order table tw; entries i = tid, tid + nthr, ...
     __host__ __device__ static __forceinline__ void fill_tables(float2* twA, float2* twB, const float2* tw, int tid,
                                                                 int nthr) {

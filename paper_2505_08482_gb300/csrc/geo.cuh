@@ -16,7 +16,7 @@ struct Geo {
     const float2* twA;   // per-layout twiddles of the split-axis passes (fft2l.cuh), or null
     const float2* twB;
     const float* kappa_t;
-    const float* kd;
+    const float2* md;
     const float2* fx;
     const float2* fy;
     const float* a_cell;
@@ -24,6 +24,7 @@ struct Geo {
     const int* srow;
     const int2* sent;
     const float4* sentw;
+    int sms;             // SMs of the device
     const int* kinst;    // instance of each data set (selects its c)
     int* status;         // workspace status word of bounded waits (nullptr: not reported)
 };
@@ -33,10 +34,11 @@ inline Geo geo(const pat_plan_s* p) {
     g.ng = p->ng; g.hc = p->hc; g.hp = p->hp; g.n = p->n; g.P = p->P; g.K = p->K; g.nt = p->nt; g.m = p->m;
     g.s_eff = p->s_eff;
     g.fft = p->fft;
-    g.tw = p->t.tw; g.twA = p->t.twA; g.twB = p->t.twB; g.kappa_t = p->t.kappa_t; g.kd = p->t.kd; g.fx = p->t.fx; g.fy = p->t.fy;
+    g.tw = p->t.tw; g.twA = p->t.twA; g.twB = p->t.twB; g.kappa_t = p->t.kappa_t; g.md = p->t.md; g.fx = p->t.fx; g.fy = p->t.fy;
     g.a_cell = p->t.a_cell; g.a_stag = p->t.a_stag;
     g.srow = p->t.srow; g.sent = p->t.sent; g.sentw = p->t.sentw;
     g.kinst = p->t.kinst;
+    g.sms = p->sms;
     g.status = nullptr;
     return g;
 }

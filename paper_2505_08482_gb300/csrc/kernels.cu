@@ -645,7 +645,6 @@ int launch_forward_cluster(const Launch& L, const Ws& w, const float* p0, const 
         set_error("no cluster-resident stepping for grid side %d", p->ng);
         return PAT_EINVAL;
     }
-    const double nrm = double(p->ng) * p->ng;
     ClusterArgs a;
     a.cg = w.cg;
     a.p0 = p0;
@@ -659,8 +658,8 @@ int launch_forward_cluster(const Launch& L, const Ws& w, const float* p0, const 
     a.n0 = n0;
     a.n1 = n1;
     a.init = state ? 0 : 1;
-    a.sg = float(p->g.dt / p->g.rho0 / nrm);
-    a.sd = float(p->g.dt * p->g.rho0 / nrm);
+    a.sg = scale_g(p);
+    a.sd = scale_d(p);
     count_launch();
     int rc = p->clops->forward(geo_ws(p, w), L.st, a);
     if (rc != PAT_OK) return rc;
@@ -674,7 +673,6 @@ int launch_forward_persistent(const Launch& L, const Ws& w, const float* p0, flo
         set_error("no persistent sweep for grid side %d", p->ng);
         return PAT_EINVAL;
     }
-    const double nrm = double(p->ng) * p->ng;
     SweepArgs a;
     a.A = w.A;
     a.B = w.B;
@@ -689,8 +687,8 @@ int launch_forward_persistent(const Launch& L, const Ws& w, const float* p0, flo
     a.last0 = last0;
     a.ckpt = ckpt;
     a.s = p->s_eff;
-    a.sg = float(p->g.dt / p->g.rho0 / nrm);
-    a.sd = float(p->g.dt * p->g.rho0 / nrm);
+    a.sg = scale_g(p);
+    a.sd = scale_d(p);
     a.nsteps = p->nt - 1;
     a.queue = w.queue;
     a.wait_ns = kQueueWaitNs;

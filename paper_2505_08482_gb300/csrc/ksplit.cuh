@@ -17,7 +17,7 @@
 // that the inverse transform of to_real needs no factor) and u lines FFT(rho0 u) / sqrt(N); then G and
 // D have the same multiplier, M = dt N^{-3/2} i k kappa exp(+-i k dx/2), without rho0, and so have the
 // adjoint's G and D with rho lines FFT(rb), u lines FFT(ub / rho0) / sqrt(N) and q lines FFT(q) / N.
-// The factor dt N^{-3/2} kappa is one table, rounded once from FP64 (a factor rounded by itself would
+// The multiplier is one table, rounded once from FP64 (a factor rounded by itself would
 // put the same relative error on every mode of every step, a wrong speed of sound), and corrected for
 // the mean gain of the three float transform pairs of a step (pair_gain: up to 7e-8 per pair, from the
 // rounded transform constants).
@@ -32,6 +32,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <type_traits>
@@ -133,21 +134,34 @@ __device__ __forceinline__ void cp16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // A tile of 2 PP columns (axis 0: [N][2 PP]) or rows (axis 1: [2 PP][S]) of a real field into shared
-// memory; x0, y0: its first column or row.  Rows of a multiple of 4 floats are copied by 16 bytes.
-template <int N, int PP, int S, int AX>
-__device__ __forceinline__ void stage_tile(float* dst, const float* f, int p0, int nt) {
+// memory, from column or row p0 on.  Rows of a multiple of 4 floats are copied by 16 bytes.  A thread's
+// pieces lie at constant distances, so that a piece is one instruction.
+template <int N, int PP, int S, int NT, int AX>
+__device__ __forceinline__ void stage_tile(float* dst, const float* f, int p0) {
     constexpr int V = (N % 4 == 0 && (2 * PP) % 4 == 0) ? 4 : 2;
-    constexpr int per = AX ? N / V : 2 * PP / V;   // pieces per row of the tile
-    const int rows = AX ? min(2 * PP, N - p0) : N;
-    for (int i = threadIdx.x; i < rows * per; i += nt) {
-        const int r = i / per, x = (i - r * per) * V;
-        if (!AX && p0 + x >= N) continue;
-        const float* src = AX ? f + size_t(p0 + r) * N + x : f + size_t(r) * N + p0 + x;
-        float* d = AX ? dst + r * S + x : dst + r * (2 * PP) + x;
+    auto piece = [](float* d, const float* src) {
         if constexpr (V == 4)
             cp16(d, src);
         else
             *reinterpret_cast<float2*>(d) = __ldcg(reinterpret_cast<const float2*>(src));
+    };
+    if constexpr (AX == 1) {
+        const int rows = min(2 * PP, N - p0);
+        for (int x = V * threadIdx.x; x < N; x += V * NT)
+            static_for<0, 2 * PP>([&](auto R) {
+                constexpr int r = decltype(R)::value;
+                if (r < rows) piece(dst + r * S + x, f + size_t(p0) * N + x + size_t(r) * N);
+            });
+    } else {
+        constexpr int per = 2 * PP / V, step = NT / per, steps = (N + step - 1) / step;
+        static_assert(NT % per == 0, "whole rows per step");
+        const int x = (threadIdx.x % per) * V, y0 = threadIdx.x / per;
+        if (p0 + x < N)
+            static_for<0, steps>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                if ((i + 1) * step <= N || y0 + i * step < N)
+                    piece(dst + (y0 + i * step) * (2 * PP) + x, f + size_t(y0) * N + p0 + x + size_t(i) * step * N);
+            });
     }
 }
 
@@ -217,16 +231,32 @@ __global__ void __launch_bounds__(PP * Fft2<N1, N2>::T) ks_to_lines(Geo g, ToLin
     const int y0 = 2 * q0;
     const bool gather = !ADJ && axis == 1 && a.y != nullptr && (mode == SP_PRESSURE || mode == SP_INIT);
     int e0 = 0, e1 = 0;
+    int2 se = make_int2(0, 0);     // the thread's first entry and its medium, fetched before the wait
+    float4 sw = make_float4(0.f, 0.f, 0.f, 0.f);
+    float c0 = 0.f, c1 = 0.f;
+    auto entry = [&](int e) {
+        se = g.sent[e];
+        sw = g.sentw[e];
+        const bool in = in_range(int(sw.w) - y0, 2 * PP, g.status) && in_range(se.y + 1, N, g.status) &&
+                        in_range(se.x, g.m, g.status) && in_range(a.tstep, g.nt, g.status);
+        if (!in) sw = make_float4(0.f, 0.f, 0.f, -1.f);
+        if (in && mode == SP_PRESSURE) {
+            const float* m = med + size_t(int(sw.w)) * N + se.y;
+            c0 = m[0];
+            c1 = m[1];
+        }
+    };
     if (gather) {
         e0 = g.srow[y0] + int(threadIdx.x);
         e1 = g.srow[min(y0 + 2 * PP, N)];
+        if (e0 < e1) entry(e0);
     }
     pdl_wait_then_release();
     if (mode == SP_PRESSURE || mode == SP_ADJOINT) {
         for_axis([&](auto A) {
             constexpr int AX = decltype(A)::value;
-            stage_tile<N, PP, S, AX>(T0, a.f0[0] + kf, y0, NT);
-            stage_tile<N, PP, S, AX>(T1, a.f0[1] + kf, y0, NT);
+            stage_tile<N, PP, S, NT, AX>(T0, a.f0[0] + kf, y0);
+            stage_tile<N, PP, S, NT, AX>(T1, a.f0[1] + kf, y0);
         });
         cp_wait_all();
     }
@@ -247,7 +277,7 @@ __global__ void __launch_bounds__(PP * Fft2<N1, N2>::T) ks_to_lines(Geo g, ToLin
                         t = make_float2(T0[2 * c * S + pos] + T1[2 * c * S + pos],
                                         T0[(2 * c + 1) * S + pos] + T1[(2 * c + 1) * S + pos]);
                     }
-                    v[n1] = make_float2(cc[n1].x * cc[n1].x * t.x, cc[n1].y * cc[n1].y * t.y);
+                    v[n1] = cprod(cprod(cc[n1], cc[n1]), t);
                     if constexpr (ADJ && AX == 1) {   // sum_n p^n pb (one addition per cell and step); 2 / c at the end
                         const int xd = pos - g.P;
                         if (ok && xd >= 0 && xd < g.n) {
@@ -290,23 +320,24 @@ __global__ void __launch_bounds__(PP * Fft2<N1, N2>::T) ks_to_lines(Geo g, ToLin
     }
     if (gather) {
         for (int e = e0; e < e1; e += NT) {
-            const int2 se = g.sent[e];
-            const float4 sw = g.sentw[e];
+            if (e != e0) entry(e);
             const int row = int(sw.w);
-            if (!(in_range(row - y0, 2 * PP, g.status) && in_range(se.y + 1, N, g.status) &&
-                  in_range(se.x, g.m, g.status) && in_range(a.tstep, g.nt, g.status)))
-                continue;
-            auto pv = [&](int x) {
-                if (mode == SP_INIT) {
-                    const int xd = x - g.P, yy = row - g.P;
-                    return (xd >= 0 && xd < g.n && yy >= 0 && yy < g.n) ? a.p0[(size_t(k) * g.n + yy) * g.n + xd] : 0.f;
-                }
-                const float cv = med[size_t(row) * N + x];
-                return cv * cv * (T0[(row - y0) * S + x] + T1[(row - y0) * S + x]);
-            };
-            const float s = sw.z * (sw.x * pv(se.y) + sw.y * pv(se.y + 1));
+            if (row < 0) continue;
+            float p0v, p1v;
+            if (mode == SP_INIT) {
+                const int xd = se.y - g.P, yy = row - g.P;
+                auto at = [&](int xv) {
+                    return (xv >= 0 && xv < g.n && yy >= 0 && yy < g.n) ? a.p0[(size_t(k) * g.n + yy) * g.n + xv] : 0.f;
+                };
+                p0v = at(xd);
+                p1v = at(xd + 1);
+            } else {
+                const int o = (row - y0) * S + se.y;
+                p0v = c0 * c0 * (T0[o] + T1[o]);
+                p1v = c1 * c1 * (T0[o + 1] + T1[o + 1]);
+            }
             // at most two adds (rows iy, iy+1) onto a zeroed sample: order-independent
-            atomicAdd(&a.y[(size_t(k) * g.nt + a.tstep) * g.m + se.x], s);
+            atomicAdd(&a.y[(size_t(k) * g.nt + a.tstep) * g.m + se.x], sw.z * (sw.x * p0v + sw.y * p1v));
         }
     }
     __syncthreads();   // the staged tiles are read: Z takes their place
@@ -405,10 +436,13 @@ __global__ void __launch_bounds__(PP * Fft2<N1, N2>::T) ks_to_real(Geo g, ToReal
     pdl_wait_then_release();
     if (!a.zero) {
         const float2* in = (blockIdx.z ? a.in1 : a.in0) + (size_t(axis) * g.K + k) * H * N + 2 * q0;
-        for (int i = threadIdx.x; i < H * PP; i += NT) {
-            const int cq = i % PP, m = i / PP;
-            if (q0 + cq < N / 2) cp16(W + i, in + size_t(m) * N + 2 * cq);
-        }
+        constexpr int step = NT / PP, steps = (H + step - 1) / step;
+        if (ok)
+            static_for<0, steps>([&](auto I) {
+                constexpr int i = decltype(I)::value;
+                if ((i + 1) * step <= H || idx + i * step < H)
+                    cp16(W + threadIdx.x + i * NT, in + size_t(idx) * N + 2 * c + size_t(i) * step * N);
+            });
         cp_wait_all();
     }
     __syncthreads();   // twiddles, source rows, staged lines
@@ -465,15 +499,13 @@ __global__ void __launch_bounds__(PP * Fft2<N1, N2>::T) ks_to_real(Geo g, ToReal
 // ---------------------------------------------------------------------------
 // the lines pass: LL lines per CTA, T threads each.  The lines' state (into shared memory, by
 // asynchronous copies), the multipliers (into the registers of the threads that use them, for both
-// operators) and the tables are fetched before the dependency wait.  The state in registers instead
-// made the pass no faster by itself but left no registers for the next pass's CTAs, whose prologue
-// then no longer overlapped.
+// operators), the twiddles (likewise: one set for all four transforms, whose twiddles all sit on the
+// A side) and the PML factors are fetched before the dependency wait.
 template <class F, int LL>
 struct LinesSmem {
     static constexpr int ZR = RowPad<F::N1, F::N2>::zs;
     static_assert(ZR >= F::ZS, "padded stride");
-    static constexpr size_t bytes =
-        size_t(2 * F::N + 2 * LL * F::N + 2 * LL * ZR) * sizeof(float2) + size_t(2) * F::N * sizeof(float);
+    static constexpr size_t bytes = size_t(2 * LL * F::N + 2 * LL * ZR) * sizeof(float2) + size_t(2) * F::N * sizeof(float);
 };
 
 template <int N1, int N2, int LL, bool ADJ>
@@ -481,9 +513,7 @@ __global__ void __launch_bounds__(LL * Fft2<N1, N2>::T) ks_lines(Geo g, LinesArg
     using F = Fft2<N1, N2>;
     constexpr int N = F::N, T = F::T, H = N / 2 + 1, NT = LL * T, ZR = LinesSmem<F, LL>::ZR;
     extern __shared__ float2 sm[];
-    float2* twA = sm;
-    float2* twB = twA + N;
-    float2* SU = twB + N;             // staged u and rho lines [LL][N]
+    float2* SU = sm;                  // staged u and rho lines [LL][N]
     float2* SR = SU + LL * N;
     float2* Z0 = SR + LL * N;
     float2* Z1 = Z0 + LL * ZR;
@@ -495,26 +525,25 @@ __global__ void __launch_bounds__(LL * Fft2<N1, N2>::T) ks_lines(Geo g, LinesArg
     const bool ok = l < lines;
     const bool aact = ok && idx < N2, bact = ok && idx < N1;
     const size_t base = size_t(l) * N + idx;
-    float2 m[N2];
+    float2 m[N2], w[N1];
     if (a.mode != SP_DIV) {   // the CTA's lines are contiguous
-        const size_t o0 = size_t(blockIdx.x) * LL * N;
+        const size_t o0 = size_t(blockIdx.x) * LL * N + 2 * threadIdx.x;
         const int pieces = min(LL, lines - int(blockIdx.x) * LL) * (N / 2);
-        for (int i = threadIdx.x; i < pieces; i += NT) {
-            cp16(SR + 2 * i, a.r + o0 + 2 * i);
-            if (a.mode != SP_STEP_FIRST) cp16(SU + 2 * i, a.u + o0 + 2 * i);
-        }
-    }
-    if (bact) {   // M at the bins idx + N1 k2 of the line's row of the table
-        const float* kd = g.kd + size_t(l % H) * N + idx;
-        const float2* f = g.fy + idx;
-        static_for<0, N2>([&](auto I) {
-            constexpr int k2 = decltype(I)::value;
-            m[k2] = cscale(f[N1 * k2], kd[N1 * k2]);
+        static_for<0, (LL * N / 2 + NT - 1) / NT>([&](auto I) {
+            constexpr int i = decltype(I)::value * NT;
+            if (int(threadIdx.x) + i < pieces) {
+                cp16(SR + 2 * threadIdx.x + 2 * i, a.r + o0 + 2 * i);
+                if (a.mode != SP_STEP_FIRST) cp16(SU + 2 * threadIdx.x + 2 * i, a.u + o0 + 2 * i);
+            }
         });
     }
+    if (bact) {   // M at the bins idx + N1 k2 of the line's row of the table
+        const float2* md = g.md + size_t(l % H) * N + idx;
+        static_for<0, N2>([&](auto I) { m[decltype(I)::value] = md[N1 * decltype(I)::value]; });
+    }
+    if (aact)
+        static_for<1, N1>([&](auto I) { w[decltype(I)::value] = g.twA[decltype(I)::value * N2 + idx]; });
     for (int i = threadIdx.x; i < N; i += NT) {
-        twA[i] = g.twA[i];
-        twB[i] = g.twB[i];
         AC[i] = g.a_cell[i];
         AS[i] = g.a_stag[i];
     }
@@ -528,7 +557,7 @@ __global__ void __launch_bounds__(LL * Fft2<N1, N2>::T) ks_lines(Geo g, LinesArg
     __syncthreads();   // tables, staged state
     // IFFT(M FFT(v)); D: M -> -conj M
     auto apply = [&](auto div) {
-        if (aact) F::fwd_a_t(v, idx, Z0 + r * ZR, twA);
+        if (aact) F::fwd_a_w(v, idx, Z0 + r * ZR, w);
         __syncthreads();
         if (bact) {
             float2 b[N2];
@@ -539,11 +568,11 @@ __global__ void __launch_bounds__(LL * Fft2<N1, N2>::T) ks_lines(Geo g, LinesArg
                 const float2 mm = decltype(div)::value ? make_float2(-m[k2].x, m[k2].y) : m[k2];
                 b[k2] = cmul(b[k2], mm);
             });
-            F::inv_b_t(b, idx, Z1 + r * ZR, twB);
+            F::inv_b_w(b, idx, Z1 + r * ZR);
         }
         __syncthreads();
         if (aact) {
-            F::inv_a_load(v, idx, Z1 + r * ZR);
+            F::inv_a_load_w(v, idx, Z1 + r * ZR, w);
             F::inv_a(v);
         }
     };
@@ -594,6 +623,19 @@ __global__ void __launch_bounds__(LL * Fft2<N1, N2>::T) ks_lines(Geo g, LinesArg
 }
 
 // ---------------------------------------------------------------------------
+// Shared memory a CTA asks for: at least a fixed slot of the SM while a launch has few CTAs per SM.
+// The CTAs of a pass are placed while those of the pass before still run (programmatic dependent launch), wherever
+// they fit; with small requests some SMs took several times their share and the pass ended with them.  With slots
+// of one size for all three passes an SM holds at most `slots` CTAs of any mix, which is every SM's share.
+// Ng 300, K = 8 (608 CTAs on 152 SMs): 17.7 us per forward step against 21.9 without slots, gradient step 50.0
+// against 54.1; K = 4 12.7 against 17.4; Ng 180, K = 16 (five slots) 14.0 against 15.5.  Beyond five CTAs per SM a
+// launch has waves enough to even out, and the slots would cost occupancy (Ng 180, K = 64: 41.8 free, 54.3 in four).
+inline size_t slot_bytes(int ctas, int sms) {
+    const int share = (ctas + sms - 1) / sms;
+    if (share > 5) return 0;
+    return share > 4 ? 38 * 1024 : 46 * 1024;   // five, four slots of an SM's 228 KB (1 KB per CTA reserved)
+}
+
 // PP pairs per CTA in the pair passes, LL lines per CTA in the lines pass
 template <int N1, int N2, int PP, int LL>
 struct SplitImpl {
@@ -603,6 +645,13 @@ struct SplitImpl {
     static constexpr size_t smem_tl = PairSmem<F, PP>::to_lines, smem_tr = PairSmem<F, PP>::to_real,
                             smem_src = PairSmem<F, PP>::source;
     static constexpr size_t smem_ln = LinesSmem<F, LL>::bytes;
+
+    // request of a pass that needs `need` bytes: the slot, or a larger one where the lines need it
+    static size_t request(const Geo& g, size_t need) {
+        const int ctas = std::max(2 * ((N / 2 + PP - 1) / PP) * g.K, (2 * g.K * H + LL - 1) / LL);
+        const size_t slot = slot_bytes(ctas, g.sms);
+        return slot ? std::max({need, slot, smem_ln}) : need;
+    }
 
     // Every forward/inverse pair in float multiplies a line by 1 + gain on average, because the
     // rounded transform constants are not exactly unitary: the mean over pseudo-random lines of
@@ -662,7 +711,8 @@ struct SplitImpl {
             {(const void*)ks_to_real<N1, N2, PP>, smem_tr + smem_src},
             {(const void*)ks_lines<N1, N2, LL, false>, smem_ln}, {(const void*)ks_lines<N1, N2, LL, true>, smem_ln}};
         for (const auto& k : ks) {
-            const cudaError_t e = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(k.b));
+            const cudaError_t e = cudaFuncSetAttribute(k.f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       int(std::max({k.b, size_t(46 * 1024), smem_ln})));
             if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute(split-axis passes)");
         }
         return PAT_OK;
@@ -670,20 +720,20 @@ struct SplitImpl {
     static dim3 pair_grid(const Geo& g, int fields) { return dim3(2 * ((N / 2 + PP - 1) / PP), g.K, fields); }
     static void to_lines(const Geo& g, cudaStream_t st, const ToLinesArgs& a, int fields, bool pdl) {
         if (a.mode == SP_ADJOINT)
-            launch_pdl(ks_to_lines<N1, N2, PP, true>, pair_grid(g, 1), dim3(PP * F::T), smem_tl, st, pdl, g, a);
+            launch_pdl(ks_to_lines<N1, N2, PP, true>, pair_grid(g, 1), dim3(PP * F::T), request(g, smem_tl), st, pdl, g, a);
         else
-            launch_pdl(ks_to_lines<N1, N2, PP, false>, pair_grid(g, fields), dim3(PP * F::T), smem_tl, st, pdl, g, a);
+            launch_pdl(ks_to_lines<N1, N2, PP, false>, pair_grid(g, fields), dim3(PP * F::T), request(g, smem_tl), st, pdl, g, a);
     }
     static void lines(const Geo& g, cudaStream_t st, const LinesArgs& a) {
         const dim3 grid((2 * g.K * H + LL - 1) / LL);
         if (a.mode == SP_STEP_ADJOINT || a.mode == SP_DIV)
-            launch_pdl(ks_lines<N1, N2, LL, true>, grid, dim3(LL * F::T), smem_ln, st, true, g, a);
+            launch_pdl(ks_lines<N1, N2, LL, true>, grid, dim3(LL * F::T), request(g, smem_ln), st, true, g, a);
         else
-            launch_pdl(ks_lines<N1, N2, LL, false>, grid, dim3(LL * F::T), smem_ln, st, true, g, a);
+            launch_pdl(ks_lines<N1, N2, LL, false>, grid, dim3(LL * F::T), request(g, smem_ln), st, true, g, a);
     }
     static void to_real(const Geo& g, cudaStream_t st, const ToRealArgs& a, int fields) {
-        launch_pdl(ks_to_real<N1, N2, PP>, pair_grid(g, fields), dim3(PP * F::T), smem_tr + (a.resid ? smem_src : 0), st,
-                   true, g, a);
+        launch_pdl(ks_to_real<N1, N2, PP>, pair_grid(g, fields), dim3(PP * F::T),
+                   request(g, smem_tr + (a.resid ? smem_src : 0)), st, true, g, a);
     }
     static SplitOps ops() { return SplitOps{N, N1, N2, &pair_gain, &configure, &to_lines, &lines, &to_real}; }
 };

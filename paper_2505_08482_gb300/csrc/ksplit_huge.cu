@@ -5,9 +5,9 @@ namespace pat {
 
 const SplitOps* split_ops_huge(int ng) {
     switch (ng) {
-        case 360: { static const SplitOps o = SplitImpl<18, 20, 4, 8>::ops(); return &o; }
-        case 384: { static const SplitOps o = SplitImpl<16, 24, 4, 8>::ops(); return &o; }
-        case 400: { static const SplitOps o = SplitImpl<20, 20, 4, 8>::ops(); return &o; }
+        case 360: { static const SplitOps o = SplitImpl<18, 20, 4, 4>::ops(); return &o; }
+        case 384: { static const SplitOps o = SplitImpl<16, 24, 4, 4>::ops(); return &o; }
+        case 400: { static const SplitOps o = SplitImpl<20, 20, 4, 4>::ops(); return &o; }
         default: return nullptr;
     }
 }

@@ -5,11 +5,11 @@ namespace pat {
 
 const SplitOps* split_ops_mid(int ng) {
     switch (ng) {
-        case 120: { static const SplitOps o = SplitImpl<10, 12, 4, 8>::ops(); return &o; }
-        case 128: { static const SplitOps o = SplitImpl<8, 16, 4, 8>::ops(); return &o; }
-        case 144: { static const SplitOps o = SplitImpl<12, 12, 4, 8>::ops(); return &o; }
-        case 150: { static const SplitOps o = SplitImpl<10, 15, 4, 8>::ops(); return &o; }
-        case 160: { static const SplitOps o = SplitImpl<10, 16, 4, 8>::ops(); return &o; }
+        case 120: { static const SplitOps o = SplitImpl<10, 12, 4, 4>::ops(); return &o; }
+        case 128: { static const SplitOps o = SplitImpl<8, 16, 4, 4>::ops(); return &o; }
+        case 144: { static const SplitOps o = SplitImpl<12, 12, 4, 4>::ops(); return &o; }
+        case 150: { static const SplitOps o = SplitImpl<10, 15, 4, 4>::ops(); return &o; }
+        case 160: { static const SplitOps o = SplitImpl<10, 16, 4, 4>::ops(); return &o; }
         default: return nullptr;
     }
 }

@@ -5,10 +5,10 @@ namespace pat {
 
 const SplitOps* split_ops_xl(int ng) {
     switch (ng) {
-        case 256: { static const SplitOps o = SplitImpl<16, 16, 4, 8>::ops(); return &o; }
-        case 270: { static const SplitOps o = SplitImpl<15, 18, 4, 8>::ops(); return &o; }
-        case 288: { static const SplitOps o = SplitImpl<16, 18, 4, 8>::ops(); return &o; }
-        case 300: { static const SplitOps o = SplitImpl<15, 20, 4, 8>::ops(); return &o; }
+        case 256: { static const SplitOps o = SplitImpl<16, 16, 4, 4>::ops(); return &o; }
+        case 270: { static const SplitOps o = SplitImpl<15, 18, 4, 4>::ops(); return &o; }
+        case 288: { static const SplitOps o = SplitImpl<16, 18, 4, 4>::ops(); return &o; }
+        case 300: { static const SplitOps o = SplitImpl<15, 20, 4, 4>::ops(); return &o; }
         default: return nullptr;
     }
 }

@@ -44,7 +44,8 @@ struct Tables {
     float2* twA;       // [ng] each: the twiddles of the split-axis passes in the order of their two
     float2* twB;       // transform steps (null: no split-axis passes for this side)
     float* kappa_t;    // [hc][ng] kappa(kx, ky) at kx * ng + ky
-    float* kd;         // [hc][ng] kappa dt ng^{-3/2}, corrected for the transforms' gain (split-axis passes, or null)
+    float2* md;        // [hc][ng] multipliers dt ng^{-3/2} i k kappa exp(i k dx/2) of the split-axis passes, corrected
+                       // for the transforms' gain (or null)
     float2* fx;        // [hc] i kx exp(+i kx dx/2)   (x factor of G; D uses -conj)
     float2* fy;        // [ng] i ky exp(+i ky dx/2)   (y factor of G; D uses -conj)
     float* a_cell;     // [ng] PML factor at cell centres
@@ -109,6 +110,8 @@ struct pat_plan_s {
     // host bookkeeping: the workspace whose history holds the last segment
     const void* hist_valid_ws;
     int device;
+    int sms;           // SMs of the device
+    double gain;       // mean gain of a float transform pair (SplitOps::pair_gain; 0 for other sides)
     // captured CUDA graphs of whole calls, keyed by call kind, buffers and variant;
     // at most kMaxGraphs are kept, the least recently replayed one is dropped first
     static constexpr size_t kMaxGraphs = 16;
@@ -209,6 +212,11 @@ bool split_factors(int ng, int* n1, int* n2, double* gain);   // gain: SplitOps:
 int split_configure(const SplitOps* ops);
 
 // ---- api.cu internals ----
+// dt/rho0 G and dt rho0 D of the four-pass step with the inverse 2-D FFT normalisation folded in, corrected for the
+// mean gain of the float transforms (two pairs in each, SplitOps::pair_gain); the second factor also makes
+// up for the rounding of the first, since their product sets the speed of sound.
+float scale_g(const pat_plan_s* p);
+float scale_d(const pat_plan_s* p);
 // Forward sweep into y [K][nt][m] with workspace regions w (checkpoints kept if keep).
 // allow_split = false: the four-pass step (a workspace too small for the split-axis passes).
 int forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y, const Ws& w, bool keep,

@@ -302,7 +302,10 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     p->graph_clock = 0;
     p->side = nullptr;
     p->ev_start = p->ev_rec[0] = p->ev_rec[1] = p->ev_adj[0] = p->ev_adj[1] = nullptr;
-    cudaGetDevice(&p->device);
+    p->sms = 0;
+    if (cudaGetDevice(&p->device) == cudaSuccess)
+        cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
+    p->sms = std::max(p->sms, 1);
     radix_schedule(ng, &p->fft);
 
     // ---- FP64 tables ----
@@ -323,6 +326,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     int f1 = 0, f2 = 0;
     double gain = 0.0;
     const bool split = split_factors(ng, &f1, &f2, &gain);
+    p->gain = split ? gain : 0.0;
     if (split) {
         twA.resize(ng);
         twB.resize(ng);
@@ -338,7 +342,13 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     };
     for (int i = 0; i < p->hc; ++i) fx[i] = gfac(k1[i], i == ng / 2);
     for (int i = 0; i < ng; ++i) fy[i] = gfac(k1[i], i == ng / 2);
-    std::vector<float> kap(size_t(p->hc) * ng), kd(split ? kap.size() : 0);
+    std::vector<float> kap(size_t(p->hc) * ng);
+    std::vector<float2> md(split ? kap.size() : 0);
+    std::vector<double> sdx(ng), cdx(ng);
+    for (int i = 0; i < ng; ++i) {
+        sdx[i] = std::sin(0.5 * k1[i] * dx);
+        cdx[i] = std::cos(0.5 * k1[i] * dx);
+    }
     // three transform pairs per step share the correction between G and D
     const double kscale = dt / (ng * std::sqrt(double(ng))) * std::pow(1.0 + gain, -1.5);
     for (int kx = 0; kx < p->hc; ++kx)
@@ -347,7 +357,10 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
             double a = 0.5 * g->c_ref * kk * dt;
             const double v = a == 0.0 ? 1.0 : std::sin(a) / a;
             kap[size_t(kx) * ng + ky] = float(v);
-            if (split) kd[size_t(kx) * ng + ky] = float(kscale * v);
+            if (split) {   // along axis ky of the line kx (either axis)
+                const double k = k1[ky], m = kscale * v * k;
+                md[size_t(kx) * ng + ky] = make_float2(float(-m * sdx[ky]), ky == ng / 2 ? 0.f : float(m * cdx[ky]));
+            }
         }
     std::vector<float> ac(ng), as(ng);
     for (int i = 0; i < ng; ++i) {
@@ -397,7 +410,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     // ---- one device allocation for all tables ----
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
-    size_t o_kd = take(kd.size() * sizeof(float)), o_ta = take(twA.size() * sizeof(float2)), o_tb = take(twB.size() * sizeof(float2));
+    size_t o_md = take(md.size() * sizeof(float2)), o_ta = take(twA.size() * sizeof(float2)), o_tb = take(twB.size() * sizeof(float2));
     size_t o_tw = take(ng * sizeof(float2)), o_k = take(kap.size() * sizeof(float));
     size_t o_fx = take(p->hc * sizeof(float2)), o_fy = take(ng * sizeof(float2));
     size_t o_ac = take(ng * sizeof(float)), o_as = take(ng * sizeof(float));
@@ -412,7 +425,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     }
     char* d = static_cast<char*>(p->dev);
     p->t.tw = reinterpret_cast<float2*>(d + o_tw);
-    p->t.kd = split ? reinterpret_cast<float*>(d + o_kd) : nullptr;
+    p->t.md = split ? reinterpret_cast<float2*>(d + o_md) : nullptr;
     p->t.twA = twA.empty() ? nullptr : reinterpret_cast<float2*>(d + o_ta);
     p->t.twB = twB.empty() ? nullptr : reinterpret_cast<float2*>(d + o_tb);
     p->t.kappa_t = reinterpret_cast<float*>(d + o_k);
@@ -428,7 +441,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     struct Cp { void* dst; const void* src; size_t n; } cps[] = {
         {p->t.tw, tw.data(), ng * sizeof(float2)},
         {p->t.twA, twA.data(), twA.size() * sizeof(float2)},
-        {p->t.kd, kd.data(), kd.size() * sizeof(float)},
+        {p->t.md, md.data(), md.size() * sizeof(float2)},
         {p->t.twB, twB.data(), twB.size() * sizeof(float2)},
         {p->t.kappa_t, kap.data(), kap.size() * sizeof(float)},
         {p->t.fx, fx.data(), p->hc * sizeof(float2)},
