@@ -58,40 +58,48 @@ __host__ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
     return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 // multiply by -i (forward) or +i (inverse)
-template <bool INV>
-__host__ __device__ __forceinline__ float2 rot(float2 a) {
-    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+template <bool INV, class C>
+__host__ __device__ __forceinline__ C rot(C a) {
+    return INV ? C{-a.y, a.x} : C{a.y, -a.x};
 }
+// the same in FP64, for the host's measurement of the transforms' gain
+__host__ inline double2 cadd(double2 a, double2 b) { return {a.x + b.x, a.y + b.y}; }
+__host__ inline double2 caxpy(double2 a, float s, double2 b) { return {a.x + double(s) * b.x, a.y + double(s) * b.y}; }
+__host__ inline double2 csub(double2 a, double2 b) { return {a.x - b.x, a.y - b.y}; }
+__host__ inline double2 cscale(double2 a, float s) { return {a.x * double(s), a.y * double(s)}; }
+__host__ inline double2 cmul(double2 a, float2 b) { return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x}; }
+__host__ inline double2 cmulc(double2 a, float2 b) { return {a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y}; }
 
 // a + rot(b), a - rot(b): the parts change places, so these stay scalar
-template <bool INV>
-__host__ __device__ __forceinline__ float2 crot_add(float2 a, float2 b) {
-    return INV ? make_float2(a.x - b.y, a.y + b.x) : make_float2(a.x + b.y, a.y - b.x);
+template <bool INV, class C>
+__host__ __device__ __forceinline__ C crot_add(C a, C b) {
+    return INV ? C{a.x - b.y, a.y + b.x} : C{a.x + b.y, a.y - b.x};
 }
-template <bool INV>
-__host__ __device__ __forceinline__ float2 crot_sub(float2 a, float2 b) {
+template <bool INV, class C>
+__host__ __device__ __forceinline__ C crot_sub(C a, C b) {
     return crot_add<!INV>(a, b);
 }
 
-// In-register DFT of R points: v_q <- sum_m v_m exp(-+ 2 pi i m q / R).
-template <int R, bool INV>
-__host__ __device__ __forceinline__ void dft_small(float2 (&v)[R]) {
+// In-register DFT of R points: v_q <- sum_m v_m exp(-+ 2 pi i m q / R).  C: float2, or double2 on the host (the
+// same float constants in FP64 arithmetic).
+template <int R, bool INV, class C>
+__host__ __device__ __forceinline__ void dft_small(C (&v)[R]) {
     if constexpr (R == 2) {
-        float2 a = v[0], b = v[1];
+        C a = v[0], b = v[1];
         v[0] = cadd(a, b);
         v[1] = csub(a, b);
     } else if constexpr (R == 3) {
         const float s3 = 0.86602540378443864676f;   // sin(2 pi / 3)
         const float sg = INV ? -s3 : s3;            // v1, v2 = m +- rot(s3 dif)
-        float2 sum = cadd(v[1], v[2]);
-        float2 dif = csub(v[1], v[2]);
-        float2 m = caxpy(v[0], -0.5f, sum);
+        C sum = cadd(v[1], v[2]);
+        C dif = csub(v[1], v[2]);
+        C m = caxpy(v[0], -0.5f, sum);
         v[0] = cadd(v[0], sum);
-        v[1] = make_float2(m.x + sg * dif.y, m.y - sg * dif.x);
-        v[2] = make_float2(m.x - sg * dif.y, m.y + sg * dif.x);
+        v[1] = C{m.x + sg * dif.y, m.y - sg * dif.x};
+        v[2] = C{m.x - sg * dif.y, m.y + sg * dif.x};
     } else if constexpr (R == 4) {
-        float2 a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
-        float2 c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+        C a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+        C c = cadd(v[1], v[3]), d = csub(v[1], v[3]);
         v[0] = cadd(a, c);
         v[2] = csub(a, c);
         v[1] = crot_add<INV>(b, d);
@@ -101,12 +109,12 @@ __host__ __device__ __forceinline__ void dft_small(float2 (&v)[R]) {
         const float c2 = -0.80901699437494742410f;   // cos(4 pi / 5)
         const float s1 = 0.95105651629515357212f;    // sin(2 pi / 5)
         const float s2 = 0.58778525229247312917f;    // sin(4 pi / 5)
-        float2 a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
-        float2 a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
-        float2 m1 = caxpy(caxpy(v[0], c1, a1), c2, a2);
-        float2 m2 = caxpy(caxpy(v[0], c2, a1), c1, a2);
-        float2 u1 = caxpy(cscale(b1, s1), s2, b2);
-        float2 u2 = caxpy(cscale(b1, s2), -s1, b2);
+        C a1 = cadd(v[1], v[4]), b1 = csub(v[1], v[4]);
+        C a2 = cadd(v[2], v[3]), b2 = csub(v[2], v[3]);
+        C m1 = caxpy(caxpy(v[0], c1, a1), c2, a2);
+        C m2 = caxpy(caxpy(v[0], c2, a1), c1, a2);
+        C u1 = caxpy(cscale(b1, s1), s2, b2);
+        C u2 = caxpy(cscale(b1, s2), -s1, b2);
         v[0] = cadd(cadd(v[0], a1), a2);
         v[1] = crot_add<INV>(m1, u1);
         v[4] = crot_sub<INV>(m1, u1);

@@ -57,13 +57,13 @@ __host__ __device__ __forceinline__ void static_for(F&& f) {
 }
 
 // z * W_N^E, W_N = exp(-2 pi i / N) (forward) or exp(+2 pi i / N) (inverse); E compile-time
-template <int N, int E, bool INV>
-__host__ __device__ __forceinline__ float2 twc(float2 z) {
+template <int N, int E, bool INV, class C>
+__host__ __device__ __forceinline__ C twc(C z) {
     constexpr int e = E % N;
     if constexpr (e == 0) {
         return z;
     } else if constexpr (2 * e == N) {
-        return make_float2(-z.x, -z.y);
+        return C{-z.x, -z.y};
     } else if constexpr (4 * e == N) {
         return rot<INV>(z);
     } else if constexpr (4 * e == 3 * N) {
@@ -73,21 +73,21 @@ __host__ __device__ __forceinline__ float2 twc(float2 z) {
         constexpr double a = (INV ? 2.0 : -2.0) * PI * double(e) / double(N);
         constexpr float c = float(ce_cos(a));
         constexpr float s = float(ce_sin(a));
-        return make_float2(z.x * c - z.y * s, z.x * s + z.y * c);
+        return C{z.x * c - z.y * s, z.x * s + z.y * c};
     }
 }
 
-template <int N, bool INV>
-__host__ __device__ __forceinline__ void dft(float2 (&v)[N]);
+template <int N, bool INV, class C>
+__host__ __device__ __forceinline__ void dft(C (&v)[N]);
 
 // N = A * B: DFT_A over a of v[B a + b] for each b, twiddle W_N^{b ka}, DFT_B over b
-template <int A, int B, bool INV>
-__host__ __device__ __forceinline__ void dft_ab(float2 (&v)[A * B]) {
+template <int A, int B, bool INV, class C>
+__host__ __device__ __forceinline__ void dft_ab(C (&v)[A * B]) {
     constexpr int N = A * B;
-    float2 t[N];
+    C t[N];
     static_for<0, B>([&](auto bI) {
         constexpr int b = decltype(bI)::value;
-        float2 u[A];
+        C u[A];
         static_for<0, A>([&](auto aI) { u[decltype(aI)::value] = v[B * decltype(aI)::value + b]; });
         dft<A, INV>(u);
         static_for<0, A>([&](auto kI) {
@@ -97,15 +97,15 @@ __host__ __device__ __forceinline__ void dft_ab(float2 (&v)[A * B]) {
     });
     static_for<0, A>([&](auto kI) {
         constexpr int ka = decltype(kI)::value;
-        float2 u[B];
+        C u[B];
         static_for<0, B>([&](auto bI) { u[decltype(bI)::value] = t[ka * B + decltype(bI)::value]; });
         dft<B, INV>(u);
         static_for<0, B>([&](auto kbI) { v[ka + A * decltype(kbI)::value] = u[decltype(kbI)::value]; });
     });
 }
 
-template <int N, bool INV>
-__host__ __device__ __forceinline__ void dft(float2 (&v)[N]) {
+template <int N, bool INV, class C>
+__host__ __device__ __forceinline__ void dft(C (&v)[N]) {
     if constexpr (N == 1) {
     } else if constexpr (N == 2 || N == 3 || N == 4 || N == 5) {
         dft_small<N, INV>(v);
@@ -148,11 +148,12 @@ struct Fft2 {
         });
     }
     // forward, B layout: b[n2] = Z[k1 P2 + n2] -> b[k2] = X[k1 + N1 k2]
-    template <int S = 1>
-    __host__ __device__ static __forceinline__ void fwd_b_load(float2 (&b)[N2], int k1, const float2* Z) {
+    template <int S = 1, class C>
+    __host__ __device__ static __forceinline__ void fwd_b_load(C (&b)[N2], int k1, const C* Z) {
         static_for<0, N2>([&](auto nI) { b[decltype(nI)::value] = Z[(k1 * P2 + decltype(nI)::value) * S]; });
     }
-    __host__ __device__ static __forceinline__ void fwd_b(float2 (&b)[N2]) { dft<N2, false>(b); }
+    template <class C>
+    __host__ __device__ static __forceinline__ void fwd_b(C (&b)[N2]) { dft<N2, false>(b); }
     // inverse, B layout: b[k2] = X[k1 + N1 k2] -> inverse DFT_N2, twiddle, Z[k1 P2 + n2]
     template <int S = 1>
     __host__ __device__ static __forceinline__ void inv_b(float2 (&b)[N2], int k1, float2* Z, const float2* tw) {
@@ -168,22 +169,22 @@ struct Fft2 {
     // threads of one step read consecutive entries (no shared-memory bank conflicts; the
     // natural-order table is read with stride k1 or n2 across threads):
     // twA[k1 N2 + n2] = twB[n2 N1 + k1] = W_N^{n2 k1}.  Same values, same results.
-    template <int S = 1>
-    __host__ __device__ static __forceinline__ void fwd_a_t(float2 (&a)[N1], int n2, float2* Z, const float2* twA) {
+    template <int S = 1, class C>
+    __host__ __device__ static __forceinline__ void fwd_a_t(C (&a)[N1], int n2, C* Z, const float2* twA) {
         dft<N1, false>(a);
         static_for<0, N1>([&](auto kI) {
             constexpr int k1 = decltype(kI)::value;
-            float2 v = a[k1];
+            C v = a[k1];
             if constexpr (k1 > 0) v = cmul(v, twA[k1 * N2 + n2]);
             Z[(k1 * P2 + n2) * S] = v;
         });
     }
-    template <int S = 1>
-    __host__ __device__ static __forceinline__ void inv_b_t(float2 (&b)[N2], int k1, float2* Z, const float2* twB) {
+    template <int S = 1, class C>
+    __host__ __device__ static __forceinline__ void inv_b_t(C (&b)[N2], int k1, C* Z, const float2* twB) {
         dft<N2, true>(b);
         static_for<0, N2>([&](auto nI) {
             constexpr int n2 = decltype(nI)::value;
-            float2 v = b[n2];
+            C v = b[n2];
             if constexpr (n2 > 0) v = cmulc(v, twB[n2 * N1 + k1]);
             Z[(k1 * P2 + n2) * S] = v;
         });
@@ -224,11 +225,12 @@ struct Fft2 {
     }
 
     // inverse, A layout: a[k1] = Z[k1 P2 + n2] -> inverse DFT_N1 -> a[n1] = x[n2 + N2 n1]
-    template <int S = 1>
-    __host__ __device__ static __forceinline__ void inv_a_load(float2 (&a)[N1], int n2, const float2* Z) {
+    template <int S = 1, class C>
+    __host__ __device__ static __forceinline__ void inv_a_load(C (&a)[N1], int n2, const C* Z) {
         static_for<0, N1>([&](auto kI) { a[decltype(kI)::value] = Z[(decltype(kI)::value * P2 + n2) * S]; });
     }
-    __host__ __device__ static __forceinline__ void inv_a(float2 (&a)[N1]) { dft<N1, true>(a); }
+    template <class C>
+    __host__ __device__ static __forceinline__ void inv_a(C (&a)[N1]) { dft<N1, true>(a); }
 };
 
 

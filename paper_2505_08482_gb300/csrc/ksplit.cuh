@@ -17,10 +17,10 @@
 // that the inverse transform of to_real needs no factor) and u lines FFT(rho0 u) / sqrt(N); then G and
 // D have the same multiplier, M = dt N^{-3/2} i k kappa exp(+-i k dx/2), without rho0, and so have the
 // adjoint's G and D with rho lines FFT(rb), u lines FFT(ub / rho0) / sqrt(N) and q lines FFT(q) / N.
-// The multiplier is one table, rounded once from FP64 (a factor rounded by itself would
-// put the same relative error on every mode of every step, a wrong speed of sound), and corrected for
-// the mean gain of the three float transform pairs of a step (pair_gain: up to 7e-8 per pair, from the
-// rounded transform constants).
+// The multiplier is one table, rounded once from FP64 (a factor rounded by itself would put the same
+// relative error on every mode of every step, a wrong speed of sound) and divided by the gain of the float
+// transform pairs that a mode meets (mode_gain, up to 7e-8 each): one along the line in each operator, one across the
+// lines per step.
 //
 // What bounds the passes: with few data sets the latency of the three launches (L2 round trip and the
 // chain of transforms, about ten warps per SM at 256^2, K = 8), with many the instruction issue of the
@@ -90,7 +90,7 @@ struct ToRealArgs {
 
 struct SplitOps {
     int ng, n1, n2;
-    double (*pair_gain)();   // mean gain of a forward and inverse float transform, minus 1
+    const double* (*mode_gain)();   // [ng] gain of a forward and inverse float transform per mode, minus 1
     int (*configure)();
     void (*to_lines)(const Geo&, cudaStream_t, const ToLinesArgs&, int fields, bool pdl);
     void (*lines)(const Geo&, cudaStream_t, const LinesArgs&);
@@ -653,57 +653,53 @@ struct SplitImpl {
         return slot ? std::max({need, slot, smem_ln}) : need;
     }
 
-    // Every forward/inverse pair in float multiplies a line by 1 + gain on average, because the
-    // rounded transform constants are not exactly unitary: the mean over pseudo-random lines of
-    // <x, IFFT(FFT(x))> / (N <x, x>) - 1, by the same code on the host (once per process and side).
-    static double measure_gain() {
-        static float2 tw[N], ta[N], tb[N];
+    // A forward/inverse pair in float multiplies the mode exp(2 pi i k n / N) by 1 + gain[k], because the rounded
+    // transform constants are not exactly unitary: measured with those constants in FP64 arithmetic, by the
+    // same code on the host (once per process and side, a few ms).
+    static std::vector<double> measure_gain() {
+        std::vector<float2> tw(N), ta(N), tb(N);
+        std::vector<double2> e(N), x(N), X(N), Z(F::ZS);
         for (int q = 0; q < N; ++q) {
             const double w = -2.0 * 3.14159265358979323846 * q / N;
+            e[q] = double2{std::cos(w), -std::sin(w)};
             tw[q] = make_float2(float(std::cos(w)), float(std::sin(w)));
         }
-        F::fill_tables(ta, tb, tw, 0, 1);
-        std::vector<float2> Z(F::ZS), x(N), X(N);
-        unsigned state = 12345u;
-        auto rnd = [&]() {
-            state = state * 1664525u + 1013904223u;
-            return float(int(state >> 8) - (1 << 23)) / float(1 << 23);
-        };
-        double num = 0.0, den = 0.0;
-        for (int t = 0; t < 48; ++t) {
-            for (auto& v : x) v = make_float2(rnd(), rnd());
+        F::fill_tables(ta.data(), tb.data(), tw.data(), 0, 1);
+        std::vector<double> gain(N);
+        for (int k = 0; k < N; ++k) {
             for (int n2 = 0; n2 < N2; ++n2) {
-                float2 a[N1];
-                for (int n1 = 0; n1 < N1; ++n1) a[n1] = x[N2 * n1 + n2];
-                F::fwd_a_t(a, n2, Z.data(), ta);
+                double2 a[N1];
+                for (int n1 = 0; n1 < N1; ++n1) a[n1] = e[size_t(k) * (N2 * n1 + n2) % N];
+                F::fwd_a_t(a, n2, Z.data(), ta.data());
             }
             for (int k1 = 0; k1 < N1; ++k1) {
-                float2 b[N2];
+                double2 b[N2];
                 F::fwd_b_load(b, k1, Z.data());
                 F::fwd_b(b);
                 for (int k2 = 0; k2 < N2; ++k2) X[k1 + N1 * k2] = b[k2];
             }
             for (int k1 = 0; k1 < N1; ++k1) {
-                float2 b[N2];
+                double2 b[N2];
                 for (int k2 = 0; k2 < N2; ++k2) b[k2] = X[k1 + N1 * k2];
-                F::inv_b_t(b, k1, Z.data(), tb);
+                F::inv_b_t(b, k1, Z.data(), tb.data());
             }
+            double s = 0.0;
             for (int n2 = 0; n2 < N2; ++n2) {
-                float2 a[N1];
+                double2 a[N1];
                 F::inv_a_load(a, n2, Z.data());
                 F::inv_a(a);
                 for (int n1 = 0; n1 < N1; ++n1) {
-                    const float2 o = x[N2 * n1 + n2];
-                    num += double(o.x) * a[n1].x + double(o.y) * a[n1].y;
-                    den += double(N) * (double(o.x) * o.x + double(o.y) * o.y);
+                    const double2 o = e[size_t(k) * (N2 * n1 + n2) % N];
+                    s += o.x * a[n1].x + o.y * a[n1].y;
                 }
             }
+            gain[k] = s / (double(N) * N) - 1.0;
         }
-        return num / den - 1.0;
-    }
-    static double pair_gain() {
-        static const double gain = measure_gain();
         return gain;
+    }
+    static const double* mode_gain() {
+        static const std::vector<double> gain = measure_gain();
+        return gain.data();
     }
     static int configure() {
         struct { const void* f; size_t b; } ks[] = {
@@ -735,7 +731,7 @@ struct SplitImpl {
         launch_pdl(ks_to_real<N1, N2, PP>, pair_grid(g, fields), dim3(PP * F::T),
                    request(g, smem_tr + (a.resid ? smem_src : 0)), st, true, g, a);
     }
-    static SplitOps ops() { return SplitOps{N, N1, N2, &pair_gain, &configure, &to_lines, &lines, &to_real}; }
+    static SplitOps ops() { return SplitOps{N, N1, N2, &mode_gain, &configure, &to_lines, &lines, &to_real}; }
 };
 
 }  // namespace pat

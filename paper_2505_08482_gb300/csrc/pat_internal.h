@@ -111,7 +111,7 @@ struct pat_plan_s {
     const void* hist_valid_ws;
     int device;
     int sms;           // SMs of the device
-    double gain;       // mean gain of a float transform pair (SplitOps::pair_gain; 0 for other sides)
+    double gain;       // mean gain of a float transform pair over the well-resolved modes (0: not measured)
     // captured CUDA graphs of whole calls, keyed by call kind, buffers and variant;
     // at most kMaxGraphs are kept, the least recently replayed one is dropped first
     static constexpr size_t kMaxGraphs = 16;
@@ -208,12 +208,12 @@ int split_adjoint(const Launch& L, const Ws& w, const float* r, int n_hi, int n_
                   int hbase);
 int split_adjoint_final(const Launch& L, const Ws& w, bool have_q, const float* r, const float* p0, float* grad_p0);
 const SplitOps* split_ops_for(int ng);   // nullptr: no split-axis passes for this grid side
-bool split_factors(int ng, int* n1, int* n2, double* gain);   // gain: SplitOps::pair_gain
+bool split_factors(int ng, int* n1, int* n2, const double** gain);   // gain: SplitOps::mode_gain
 int split_configure(const SplitOps* ops);
 
 // ---- api.cu internals ----
 // dt/rho0 G and dt rho0 D of the four-pass step with the inverse 2-D FFT normalisation folded in, corrected for the
-// mean gain of the float transforms (two pairs in each, SplitOps::pair_gain); the second factor also makes
+// mean gain of the float transforms (two pairs in each); the second factor also makes
 // up for the rounding of the first, since their product sets the speed of sound.
 float scale_g(const pat_plan_s* p);
 float scale_d(const pat_plan_s* p);

@@ -324,9 +324,11 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
     // the same twiddles in the order in which the two transform steps of the split-axis passes read them
     std::vector<float2> twA, twB;
     int f1 = 0, f2 = 0;
-    double gain = 0.0;
+    const double* gain = nullptr;
     const bool split = split_factors(ng, &f1, &f2, &gain);
-    p->gain = split ? gain : 0.0;
+    p->gain = 0.0;
+    if (split)   // modes up to an eighth of the sampling rate
+        for (int k = -ng / 8; k <= ng / 8; ++k) p->gain += gain[(k + ng) % ng] / (2 * (ng / 8) + 1);
     if (split) {
         twA.resize(ng);
         twB.resize(ng);
@@ -349,8 +351,7 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
         sdx[i] = std::sin(0.5 * k1[i] * dx);
         cdx[i] = std::cos(0.5 * k1[i] * dx);
     }
-    // three transform pairs per step share the correction between G and D
-    const double kscale = dt / (ng * std::sqrt(double(ng))) * std::pow(1.0 + gain, -1.5);
+    const double kscale = dt / (ng * std::sqrt(double(ng)));
     for (int kx = 0; kx < p->hc; ++kx)
         for (int ky = 0; ky < ng; ++ky) {
             double kk = std::sqrt(k1[kx] * k1[kx] + k1[ky] * k1[ky]);
@@ -358,7 +359,8 @@ extern "C" int pat_plan_create_batched(pat_plan* out, const pat_grid* g, int m, 
             const double v = a == 0.0 ? 1.0 : std::sin(a) / a;
             kap[size_t(kx) * ng + ky] = float(v);
             if (split) {   // along axis ky of the line kx (either axis)
-                const double k = k1[ky], m = kscale * v * k;
+                // the mode's transform gain: a pair along the line, half a pair across
+                const double k = k1[ky], m = kscale * v * k / ((1.0 + gain[ky]) * std::sqrt(1.0 + gain[kx]));
                 md[size_t(kx) * ng + ky] = make_float2(float(-m * sdx[ky]), ky == ng / 2 ? 0.f : float(m * cdx[ky]));
             }
         }

@@ -63,10 +63,10 @@ const SplitOps* split_ops_for(int ng) {
     return nullptr;
 }
 
-bool split_factors(int ng, int* n1, int* n2, double* gain) {
+bool split_factors(int ng, int* n1, int* n2, const double** gain) {
     const SplitOps* o = split_ops_for(ng);
     if (!o) return false;
-    *gain = o->pair_gain();
+    *gain = o->mode_gain();
     *n1 = o->n1;
     *n2 = o->n2;
     return true;
