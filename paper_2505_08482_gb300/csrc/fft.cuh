@@ -15,6 +15,10 @@ struct FftDesc {
     int n;
     int nrad;
     int rad[kMaxStages];
+    // per stage: ceil(2^32 / (n / rad)) and ceil(2^32 / Ns) (Ns: the sub-transforms already done), so that a division
+    // of the stage's indices (below 2^20) is one multiplication
+    unsigned inv_nb[kMaxStages];
+    unsigned inv_ns[kMaxStages];
 };
 
 // Additions and real factors of complex values act on both parts alike: one packed instruction
@@ -128,16 +132,16 @@ __host__ __device__ __forceinline__ void dft_small(C (&v)[R]) {
 template <int R, bool INV>
 __device__ __forceinline__ void stockham_stage(const float2* __restrict__ src, float2* __restrict__ dst,
                                                int n, int Ns, int nseq, int ss,
-                                               const float2* __restrict__ tw) {
+                                               const float2* __restrict__ tw, unsigned inv_nb, unsigned inv_ns) {
     const int nb = n / R;
     const int tstride = n / (Ns * R);
     const int total = nseq * nb;
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int s = t / nb;
+        const int s = nb > 1 ? int(__umulhi(unsigned(t), inv_nb)) : t;
         const int j = t - s * nb;
         const float2* in = src + s * ss;
         float2* out = dst + s * ss;
-        const int k = j % Ns;
+        const int k = Ns > 1 ? j - int(__umulhi(unsigned(j), inv_ns)) * Ns : 0;
         float2 v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = in[j + r * nb];
@@ -166,10 +170,10 @@ __device__ float2* fft_smem(float2* a, float2* b, int nseq, int ss, const FftDes
     for (int st = 0; st < fd.nrad; ++st) {
         const int R = fd.rad[st];
         switch (R) {
-            case 2: stockham_stage<2, INV>(a, b, fd.n, Ns, nseq, ss, tw); break;
-            case 3: stockham_stage<3, INV>(a, b, fd.n, Ns, nseq, ss, tw); break;
-            case 4: stockham_stage<4, INV>(a, b, fd.n, Ns, nseq, ss, tw); break;
-            default: stockham_stage<5, INV>(a, b, fd.n, Ns, nseq, ss, tw); break;
+            case 2: stockham_stage<2, INV>(a, b, fd.n, Ns, nseq, ss, tw, fd.inv_nb[st], fd.inv_ns[st]); break;
+            case 3: stockham_stage<3, INV>(a, b, fd.n, Ns, nseq, ss, tw, fd.inv_nb[st], fd.inv_ns[st]); break;
+            case 4: stockham_stage<4, INV>(a, b, fd.n, Ns, nseq, ss, tw, fd.inv_nb[st], fd.inv_ns[st]); break;
+            default: stockham_stage<5, INV>(a, b, fd.n, Ns, nseq, ss, tw, fd.inv_nb[st], fd.inv_ns[st]); break;
         }
         __syncthreads();
         float2* t = a;

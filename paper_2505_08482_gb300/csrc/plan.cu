@@ -53,6 +53,13 @@ bool radix_schedule(int n, FftDesc* fd) {
             r /= q;
         }
     }
+    int ns = 1;
+    for (int i = 0; i < fd->nrad; ++i) {   // nb = n / rad >= 2 wherever a stage has more than one butterfly
+        const int nb = n / fd->rad[i];
+        fd->inv_nb[i] = nb > 1 ? unsigned((0x100000000ull + nb - 1) / nb) : 0u;
+        fd->inv_ns[i] = ns > 1 ? unsigned((0x100000000ull + ns - 1) / ns) : 0u;
+        ns *= fd->rad[i];
+    }
     return r == 1;
 }
 

