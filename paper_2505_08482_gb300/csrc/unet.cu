@@ -60,6 +60,7 @@ struct pat_unet_s {
     __nv_bfloat16* wt = nullptr;         // bf16 weights with input and output channels exchanged (data gradient)
     ConvDesc* desc = nullptr;            // device copy of the convolutions' weight places
     float* bpart = nullptr;              // partial sums of the bias gradients and the head
+    unsigned* done = nullptr;            // blocks of the running bias sum that are done (0 between launches)
     const Conv* col_of = nullptr;        // the convolution whose im2col of the current input `col` holds
     __nv_bfloat16* col = nullptr;        // scratch: im2col / transposes
     __nv_bfloat16* colt = nullptr;
@@ -112,8 +113,13 @@ int conv_fwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16*
     const __nv_bfloat16* wb = u->wbf + c.wb_off;
     const float* bias = u->param + c.b_off;
     if (u->gemm_path == 1 && unet_conv_supported(in, ldin, c.cin, c.cout))
-        return unet_conv(st, in, ldin, wb, B, c.H, c.W, c.cin, c.cout, 0, bias, 1, nullptr, out, c.cout, u->status);
+        return unet_conv(st, in, ldin, wb, B, c.H, c.W, c.cin, c.cout, 9, 9 * c.cin, 0, bias, 1, nullptr, out, c.cout,
+                         u->status);
     RC(make_col(u, st, c, in, ldin, B));
+    // the padded im2col rows as a 1x1 convolution (the weights' rows end at 9 cin: zero fill)
+    if (u->gemm_path == 1 && unet_conv_supported(u->col, col_pitch(c.cin), col_pitch(c.cin), c.cout))
+        return unet_conv(st, u->col, col_pitch(c.cin), wb, B, c.H, c.W, col_pitch(c.cin), c.cout, 1, 9 * c.cin, 0, bias, 1,
+                         nullptr, out, c.cout, u->status);
     return net_gemm(u, st, u->col, col_pitch(c.cin), wb, 9 * c.cin, B * c.H * c.W, c.cout, 9 * c.cin, bias, 1, out,
                     c.cout, 0, 1);
 }
@@ -124,7 +130,7 @@ int conv_bwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16*
              const __nv_bfloat16* dz, __nv_bfloat16* din, const __nv_bfloat16* mask) {
     const int P = B * c.H * c.W, K1 = 9 * c.cin;
     float* dW = u->grad + c.w_off;
-    RC(unet_bias_grad(st, dz, u->grad + c.b_off, u->bpart, size_t(P), c.cout));
+    RC(unet_bias_grad(st, dz, u->grad + c.b_off, u->bpart, u->done, size_t(P), c.cout));
     if (u->gemm_path == 1 && unet_wgrad_supported(in, ldin, c.cin, c.cout)) {
         RC(unet_wgrad(st, in, ldin, dz, B, c.H, c.W, c.cin, 9, c.cout, dW, K1, u->status));
     } else if (u->gemm_path == 1 && unet_wgrad_supported(u->col, col_pitch(c.cin), col_pitch(c.cin), c.cout)) {
@@ -141,7 +147,8 @@ int conv_bwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16*
     // din[p][ci] = sum_{tap,co} dz[p - off(tap)][co] W[co][tap][ci]
     const __nv_bfloat16* wt = u->wt + c.wb_off;
     if (u->gemm_path == 1 && unet_conv_supported(dz, c.cout, c.cout, c.cin))
-        return unet_conv(st, dz, c.cout, wt, B, c.H, c.W, c.cout, c.cin, 1, nullptr, 0, mask, din, c.cin, u->status);
+        return unet_conv(st, dz, c.cout, wt, B, c.H, c.W, c.cout, c.cin, 9, 9 * c.cout, 1, nullptr, 0, mask, din, c.cin,
+                         u->status);
     u->col_of = nullptr;
     RC(unet_im2col(st, dz, u->col, B, c.H, c.W, c.cout, c.cout, 1, 9 * c.cout));
     RC(net_gemm(u, st, u->col, 9 * c.cout, wt, 9 * c.cout, P, c.cin, 9 * c.cout, nullptr, 0, din, c.cin, 0, 1));
@@ -311,7 +318,9 @@ extern "C" int pat_unet_create(pat_unet* out, int levels, int base, int in_ch, i
     if (rc == PAT_OK) rc = dalloc(u, &u->part, unet_part_blocks());
     if (rc == PAT_OK) rc = dalloc(u, &u->loss, 1);
     if (rc == PAT_OK) rc = dalloc(u, &u->status, 1);
-    if (rc == PAT_OK && cudaMemset(u->status, 0, sizeof(int)) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "unet status");
+    if (rc == PAT_OK) rc = dalloc(u, &u->done, 1);
+    if (rc == PAT_OK && (cudaMemset(u->status, 0, sizeof(int)) != cudaSuccess ||
+                         cudaMemset(u->done, 0, sizeof(unsigned)) != cudaSuccess)) rc = cuda_fail(cudaGetLastError(), "unet status");
     if (rc == PAT_OK) {
         std::vector<ConvDesc> d;
         for (const Conv& c : u->convs) d.push_back(ConvDesc{c.cin, c.cout, c.k, c.w_off, c.wb_off});

@@ -16,12 +16,13 @@ int unet_gemm(cudaStream_t st, const __nv_bfloat16* A, int lda, const __nv_bfloa
 bool unet_gemm_tc05_supported(const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N, int K);
 int unet_gemm_tc05(cudaStream_t st, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, int M, int N,
                    int K, const float* bias, int relu, void* C, int ldc, int out_mode, int splitk, int* d_status);
-// 3x3 convolution without im2col (unet_conv.cu): out[p][cout] (pitch ldo, bf16) = conv(in, W[cout][9][cin]) (+ bias)
+// 3x3 (taps 9) or 1x1 (taps 1) convolution without im2col (unet_conv.cu), weight rows of kw >= taps * cin or zero-
+// extended elements: out[p][cout] (pitch ldo, bf16) = conv(in, W[cout][kw]) (+ bias)
 // (ReLU) (zero where mask <= 0, pitch cout); flip: taps reversed (data gradient)
 bool unet_conv_supported(const __nv_bfloat16* in, int ldin, int cin, int cout);
 int unet_conv(cudaStream_t st, const __nv_bfloat16* in, int ldin, const __nv_bfloat16* W, int B, int H, int Wd, int cin,
-              int cout, int flip, const float* bias, int relu, const __nv_bfloat16* mask, __nv_bfloat16* out, int ldo,
-              int* d_status);
+              int cout, int taps, int kw, int flip, const float* bias, int relu, const __nv_bfloat16* mask,
+              __nv_bfloat16* out, int ldo, int* d_status);
 // dW[cout][kw] += sum_p dz[p][cout] in[p + off(tap)][c] at tap * cin + c < kw (taps 9, or 1 unshifted); dW zeroed by the caller
 bool unet_wgrad_supported(const __nv_bfloat16* in, int ldin, int cin, int cout);
 int unet_wgrad(cudaStream_t st, const __nv_bfloat16* in, int ldin, const __nv_bfloat16* dz, int B, int H, int Wd, int cin,
@@ -46,7 +47,7 @@ int unet_upsample_bwd(cudaStream_t st, const __nv_bfloat16* cat, const __nv_bflo
 int unet_relu_bwd(cudaStream_t st, __nv_bfloat16* g, const __nv_bfloat16* y, size_t n);
 size_t unet_part_floats(int C);   // scratch of the two-step sums below
 int unet_part_blocks();
-int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* part, size_t P, int C);
+int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* part, unsigned* done, size_t P, int C);
 int unet_head(cudaStream_t st, const __nv_bfloat16* y, const __nv_bfloat16* w, const float* bias, float* out, size_t P,
               int C);
 int unet_head_bwd(cudaStream_t st, const float* out, const float* tgt, const __nv_bfloat16* y, const __nv_bfloat16* w,

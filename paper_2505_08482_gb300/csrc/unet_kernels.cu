@@ -359,22 +359,31 @@ __global__ void k_relu_bwd(__nv_bfloat16* __restrict__ g, const __nv_bfloat16* _
     }
 }
 
-// Bias gradient db[c] = sum_p g[p][c], in two steps of fixed order: block (b, z) sums the pixels b, b +
-// gridDim.x, ... (in groups of 256 / G) of 8 G channels from 64 z on into part[b][C]; then one block sums the parts.
+// Bias gradient db[c] = sum_p g[p][c] in a fixed order: block (b, z) sums every gridDim.x-th group of 256 / G pixels
+// for 8 G channels from 64 z on into part[b][C], four reads in flight per thread; the block that is done last
+// sums the parts.
 constexpr int kBiasBlocks = 296;
-__global__ void __launch_bounds__(256) k_bias_part(const __nv_bfloat16* __restrict__ g, float* __restrict__ part,
-                                                   size_t P, int C) {
+__global__ void __launch_bounds__(256) k_bias_grad(const __nv_bfloat16* __restrict__ g, float* __restrict__ part,
+                                                   unsigned* __restrict__ done, float* __restrict__ db, size_t P, int C) {
     __shared__ float red[256][9];
+    __shared__ bool last;
     const int c0 = blockIdx.y * 64, G = min(8, (C - c0) / 8);
     const int R = 256 / G, cg = threadIdx.x % G, pr = threadIdx.x / G;
     float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (pr < R)
-        for (size_t p = size_t(blockIdx.x) * R + pr; p < P; p += size_t(gridDim.x) * R) {
-            Bf8 v;
-            v.u = *reinterpret_cast<const uint4*>(g + p * C + c0 + cg * 8);
+    if (pr < R) {
+        const size_t step = size_t(gridDim.x) * R;
+        const __nv_bfloat16* src = g + c0 + cg * 8;
+        for (size_t p = size_t(blockIdx.x) * R + pr; p < P; p += 4 * step) {
+            Bf8 v[4];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) s[j] += __bfloat162float(v.h[j]);
+            for (int q = 0; q < 4; ++q)
+                v[q].u = p + q * step < P ? *reinterpret_cast<const uint4*>(src + (p + q * step) * C) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s[j] += __bfloat162float(v[q].h[j]);
         }
+    }
 #pragma unroll
     for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = s[j];
     __syncthreads();
@@ -384,13 +393,34 @@ __global__ void __launch_bounds__(256) k_bias_part(const __nv_bfloat16* __restri
         for (int r = 0; r < R; ++r) t += red[r * G + c][j];
         part[size_t(blockIdx.x) * C + c0 + c * 8 + j] = t;
     }
-}
-__global__ void k_bias_sum(const float* __restrict__ part, int nblk, float* __restrict__ db, int C) {
-    const int c = blockIdx.x, lane = threadIdx.x;
-    float s = 0.f;
-    for (int b = lane; b < nblk; b += 32) s += part[size_t(b) * C + c];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) db[c] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {   // one fence for the block's parts, ordered by the barrier
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x * gridDim.y - 1;
+        if (last) *done = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    // 256 / C threads per channel (at least one), consecutive threads on consecutive channels
+    float* sum = &red[0][0];
+    const int per = max(1, 256 / C), nb = int(gridDim.x);
+    for (int cb = 0; cb < C; cb += 256) {
+        const int w = min(C - cb, 256), q = threadIdx.x / w, c = cb + threadIdx.x - q * w;
+        float t = 0.f;
+        if (q < per) {
+#pragma unroll 8
+            for (int b = q; b < nb; b += per) t += __ldcg(part + size_t(b) * C + c);
+        }
+        __syncthreads();
+        sum[threadIdx.x] = t;
+        __syncthreads();
+        if (q == 0) {
+            for (int i = 1; i < per; ++i) t += sum[i * w + threadIdx.x];
+            db[c] = t;
+        }
+        __syncthreads();
+    }
 }
 
 // Final 1x1 convolution to one channel: out[p] = sum_c y[p][c] w[c] + b.  A warp takes 16 pixels as the rows of
@@ -589,12 +619,12 @@ int unet_relu_bwd(cudaStream_t st, __nv_bfloat16* g, const __nv_bfloat16* y, siz
     LAUNCH_CHECK("k_relu_bwd");
     return PAT_OK;
 }
-int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* part, size_t P, int C) {
-    const unsigned nb = unsigned(std::min<size_t>(kBiasBlocks, (P + 31) / 32));
-    k_bias_part<<<dim3(nb, (C + 63) / 64), 256, 0, st>>>(g, part, P, C);
-    LAUNCH_CHECK("k_bias_part");
-    k_bias_sum<<<C, 32, 0, st>>>(part, int(nb), db, C);
-    LAUNCH_CHECK("k_bias_sum");
+int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* part, unsigned* done, size_t P, int C) {
+    // at least 16 pixels per thread: the last block's sum grows with the blocks
+    const size_t group = 256 / std::min(8, C / 8);
+    const unsigned nb = unsigned(std::max<size_t>(1, std::min<size_t>(kBiasBlocks, P / (16 * group))));
+    k_bias_grad<<<dim3(nb, (C + 63) / 64), 256, 0, st>>>(g, part, done, db, P, C);
+    LAUNCH_CHECK("k_bias_grad");
     return PAT_OK;
 }
 size_t unet_part_floats(int C) { return size_t(kBiasBlocks > kHeadBlocks ? kBiasBlocks : kHeadBlocks) * (C + 1); }
