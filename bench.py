@@ -45,7 +45,7 @@ WL = dict(workload="vessels256", n=256, K=8, M=512, nt=1800, ckpt_every=32, dx=1
 
 # Algorithmic bytes per grid cell (Ng^2 cells per data set) and launch, FP32.
 # A spectrum row holds Ng/2+1 complex values: 8 (Ng/2+1)/Ng bytes per cell.
-def bytes_per_cell(cls: int, ng: int, n: int, ckpt_hist: bool = True) -> float:
+def bytes_per_cell(cls: int, ng: int, n: int, ckpt_hist: bool = True, adjoint: bool = False) -> float:
     spec = 8.0 * (ng // 2 + 1) / ng
     dom = (n * n) / float(ng * ng)
     table = {
@@ -56,6 +56,11 @@ def bytes_per_cell(cls: int, ng: int, n: int, ckpt_hist: bool = True) -> float:
         5: 2 * spec + spec,                                          # col sum: 2 in, 1 out
         6: spec + 8 + 4 + 4 + 8 * dom + 8 + 2 * spec,                # adj rho: spectrum, rb r+w, c, hist, cbar r+w, 2 out
         7: 2 * spec + 8 + 8 + 2 * spec,                              # adj u
+        # split-axis step, both axes: pressure lines in, u and rho lines r+w (adjoint: q lines out)
+        8: 10 * spec + (2 * spec if adjoint else 0),
+        # two real fields, c, lines out, hist (adjoint: and cbar r+w)
+        9: 8 + 4 + 2 * spec + (4 if ckpt_hist else 0) + (8 * dom if adjoint else 0),
+        10: 2 * spec + 8,                                            # lines in, two real fields out
     }
     return table[cls]
 
@@ -66,7 +71,8 @@ def bytes_per_cell(cls: int, ng: int, n: int, ckpt_hist: bool = True) -> float:
 FWD_BYTES = 36.5
 GRAD_BYTES = 125.0
 
-KERNEL_FILES = ("fft.cuh", "fft2l.cuh", "geo.cuh", "sync.cuh", "dcheck.cuh", "kfixed.cuh", "kfixed_300.cu", "kernels.cu", "api.cu")
+KERNEL_FILES = ("fft.cuh", "fft2l.cuh", "geo.cuh", "sync.cuh", "dcheck.cuh", "kfixed.cuh", "kfixed_300.cu", "kernels.cu", "api.cu",
+                "ksplit.cuh", "ksplit_xl.cu", "split.cu")
 
 
 def kernel_source_hash() -> str:
@@ -358,23 +364,26 @@ def solo_class_times(plan, gs, sensors, c0, p0, stream, dev):
     out = {}
     y = torch.empty((K, nt, M), dtype=torch.float32, device=dev)
     plan.forward(c0, p0, y=y, stream=stream)
-    for cls in (B.PAT_K_ROW_RHO, B.PAT_K_ROW_U, B.PAT_K_COL_GRAD, B.PAT_K_COL_PAIR):
+    split = (B.PAT_K_LINES, B.PAT_K_TO_LINES, B.PAT_K_TO_REAL)
+    # the classes of the four-pass and of the split-axis step: those that the plan's variant launches
+    for cls in (B.PAT_K_ROW_RHO, B.PAT_K_ROW_U, B.PAT_K_COL_GRAD, B.PAT_K_COL_PAIR) + split:
         B.check(L.pat_timing_enable(cls, 2 * nt, 1), "pat_timing_enable")
         plan.forward(c0, p0, y=y, stream=stream)
         tot, cnt = ctypes_read(L)
-        out[(cls, "forward")] = (1e3 * tot / max(cnt, 1), cnt)
+        if cnt:
+            out[(cls, "forward")] = (1e3 * tot / cnt, cnt)
     B.check(L.pat_timing_enable(0, 0, 1), "pat_timing_enable")
     hplan = Plan(gs, sensors, K, ckpt_every=nt, device=dev)
     hplan.variant = plan.variant
     ybar = torch.full((K, nt, M), 1e-3, dtype=torch.float32, device=dev)
-    for cls in (0, B.PAT_K_COL_PAIR, B.PAT_K_COL_SUM, B.PAT_K_ROW_ADJ_RHO, B.PAT_K_ROW_ADJ_U):
+    for cls in (0, B.PAT_K_COL_PAIR, B.PAT_K_COL_SUM, B.PAT_K_ROW_ADJ_RHO, B.PAT_K_ROW_ADJ_U) + split:
         hplan.forward(c0, p0, y=y, keep_checkpoints=True, stream=stream)
         if cls:
             B.check(L.pat_timing_enable(cls, 2 * nt, 1), "pat_timing_enable")
         hplan.vjp(c0, p0, ybar, stream=stream)
         tot, cnt = ctypes_read(L)
-        if cls:
-            out[(cls, "adjoint")] = (1e3 * tot / max(cnt, 1), cnt)
+        if cls and cnt:
+            out[(cls, "adjoint")] = (1e3 * tot / cnt, cnt)
     B.check(L.pat_timing_enable(0, 0, 1), "pat_timing_enable")
     torch.cuda.synchronize()
     del hplan
@@ -602,7 +611,7 @@ def run_ours(args, rank, world, local_rank):
     serial_us = sum(solo[k][0] * phase_launches[k] for k in solo)
     dom, dom_phase = dom_key
     dom_us, dom_cnt = solo[dom_key]
-    bpl = bytes_per_cell(dom, ng, n) * ng * ng * K
+    bpl = bytes_per_cell(dom, ng, n, adjoint=dom_phase == "adjoint") * ng * ng * K
     achieved = bpl / (dom_us * 1e-6) / 1e9
     per_eval_ms = t_ms / args.steps
     cells = ng * ng * K * (nt - 1)
@@ -1064,11 +1073,14 @@ def roofline_k(K, nt, variant, ckpt, warmup, steps, cluster=False):
     torch.cuda.synchronize()
     peak, peak_kind = measured_peaks()
     passes = {}
-    for cls in (() if cluster else (3, 2, 4, 1)):     # the four passes of a forward step
+    # the passes of a forward step: four, or the three of the split-axis step
+    for cls in (() if cluster else (3, 2, 4, 1, B.PAT_K_LINES, B.PAT_K_TO_LINES, B.PAT_K_TO_REAL)):
         B.check(L.pat_timing_enable(cls, nt + 8, 1), "pat_timing_enable")
         plan.forward(c, p0, y=y, stream=stream)
         tot, cnt = ctypes_read(L)
         B.check(L.pat_timing_enable(0, 0, 1), "pat_timing_enable")
+        if not cnt:
+            continue
         bpl = bytes_per_cell(cls, ng, n, ckpt_hist=False) * ng * ng * K
         us = tot * 1000.0 / max(cnt, 1)
         passes[B.KERNEL_CLASSES[cls]] = {"launches": cnt, "avg_launch_us": round(us, 2),
