@@ -25,8 +25,8 @@
 // What bounds the passes: with few data sets the latency of the three launches (L2 round trip and the
 // chain of transforms, about ten warps per SM at 256^2, K = 8), with many the instruction issue of the
 // transforms.  Measured on GB300, us per forward step, four-pass step -> this one: Ng 108, K = 1 11.5 ->
-// 7.9; Ng 180, K = 4 14.3 -> 11.1; Ng 300, K = 8 23.3 -> 19.7; Ng 180, K = 64 64.6 -> 45.3; per gradient
-// step (Ng 300, K = 8) 65.1 -> 56.4.  A pass takes its registers and shared memory sparingly: what it
+// 7.2; Ng 180, K = 4 14.3 -> 9.9; Ng 300, K = 8 23.3 -> 17.7; Ng 180, K = 64 64.6 -> 41.8; per gradient
+// step (Ng 300, K = 8) 65.1 -> 50.0.  A pass takes its registers and shared memory sparingly: what it
 // leaves free lets the CTAs of the next pass run their prologue (programmatic dependent launch).
 #pragma once
 
