@@ -48,9 +48,11 @@ inline Geo geo(const pat_plan_s* p) {
 // attribute), then let the next kernel be scheduled.  A kernel may read data
 // written two or more kernels earlier before the wait, but data written by the
 // immediately preceding kernel only after it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_then_release() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait();
+    pdl_release();
 }
 
 // c of data set k's instance on the grid

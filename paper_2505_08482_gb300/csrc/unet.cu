@@ -130,11 +130,14 @@ int conv_bwd(pat_unet_s* u, cudaStream_t st, const Conv& c, const __nv_bfloat16*
              const __nv_bfloat16* dz, __nv_bfloat16* din, const __nv_bfloat16* mask) {
     const int P = B * c.H * c.W, K1 = 9 * c.cin;
     float* dW = u->grad + c.w_off;
+    const bool direct = u->gemm_path == 1 && unet_wgrad_supported(in, ldin, c.cin, c.cout);
+    const bool rows = !direct && u->gemm_path == 1 &&
+                      unet_wgrad_supported(u->col, col_pitch(c.cin), col_pitch(c.cin), c.cout);
+    if (rows) RC(make_col(u, st, c, in, ldin, B));
     RC(unet_bias_grad(st, dz, u->grad + c.b_off, u->bpart, u->done, size_t(P), c.cout));
-    if (u->gemm_path == 1 && unet_wgrad_supported(in, ldin, c.cin, c.cout)) {
+    if (direct) {   // (directly after the bias sum, as unet_wgrad asks)
         RC(unet_wgrad(st, in, ldin, dz, B, c.H, c.W, c.cin, 9, c.cout, dW, K1, u->status));
-    } else if (u->gemm_path == 1 && unet_wgrad_supported(u->col, col_pitch(c.cin), col_pitch(c.cin), c.cout)) {
-        RC(make_col(u, st, c, in, ldin, B));
+    } else if (rows) {
         RC(unet_wgrad(st, u->col, col_pitch(c.cin), dz, B, c.H, c.W, col_pitch(c.cin), 1, c.cout, dW, K1, u->status));
     } else {   // dW[co][k] = sum_p dz[p][co] col[p][k] from transposed operands, split K over pixels
         RC(unet_transpose(st, dz, u->dt, P, c.cout, c.cout));

@@ -23,7 +23,8 @@ bool unet_conv_supported(const __nv_bfloat16* in, int ldin, int cin, int cout);
 int unet_conv(cudaStream_t st, const __nv_bfloat16* in, int ldin, const __nv_bfloat16* W, int B, int H, int Wd, int cin,
               int cout, int taps, int kw, int flip, const float* bias, int relu, const __nv_bfloat16* mask,
               __nv_bfloat16* out, int ldo, int* d_status);
-// dW[cout][kw] += sum_p dz[p][cout] in[p + off(tap)][c] at tap * cin + c < kw (taps 9, or 1 unshifted); dW zeroed by the caller
+// dW[cout][kw] += sum_p dz[p][cout] in[p + off(tap)][c] at tap * cin + c < kw (taps 9, or 1 unshifted); dW zeroed by the caller;
+// reads in and dz without waiting for the kernel before it in the stream, which must be the bias sum of the same dz
 bool unet_wgrad_supported(const __nv_bfloat16* in, int ldin, int cin, int cout);
 int unet_wgrad(cudaStream_t st, const __nv_bfloat16* in, int ldin, const __nv_bfloat16* dz, int B, int H, int Wd, int cin,
                int taps, int cout, float* dW, int kw, int* d_status);

@@ -21,10 +21,17 @@
 // gradients 1.6 ms, against 20.5 ms of im2col, 3.5 of transposes and 4.5 of GEMMs; a 32 -> 32 convolution at full size
 // 50 us (193 TFLOP/s), its weight gradient 28 us.
 //
+// The kernels of the convolutions, the bias sums, the pooling and the concatenation are launched with programmatic
+// stream serialisation: a kernel's barriers and tensor memory are set up while the one before drains.  A CTA
+// lets the next kernel start only once it has its tensor memory, so that a later kernel's allocation never keeps an
+// earlier one waiting.  The weight gradient depends on nothing that the bias sum before it writes: it runs beside it
+// and waits for it only before its own stores.  Forward of 8 images 0.341 -> 0.293 ms, gradients of 32 2.12 -> 1.91 ms.
+//
 // Every mbarrier wait is bounded as in unet_tc05.cu: a wait that gives up sets PAT_STATUS_TC05 and the CTA
 // drains its copies, frees its tensor memory and returns without storing.
 #include <algorithm>
 
+#include "kfixed.cuh"
 #include "pat_internal.h"
 #include "tc05.cuh"
 #include "unet.h"
@@ -132,6 +139,7 @@ __global__ void __launch_bounds__(CONV_THREADS) k_conv(const __grid_constant__ C
     const int per_tap = a.cin / KB, nk = a.taps * per_tap;
     if (HALO && threadIdx.x == 0) mbar_init(input, 1);
     const uint32_t tmem = begin(ring, a.stages, a.cols);
+    pdl_wait_then_release();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0 && lane == 0) {   // producer
         if (HALO) {
@@ -254,6 +262,7 @@ __global__ void __launch_bounds__(CONV_THREADS) k_wgrad(const __grid_constant__ 
     const int na = min(NA, (a.rows - r0 + CA - 1) / CA);
     const int t0 = blockIdx.y * a.per, t1 = min(t0 + a.per, a.tiles), nk = t1 - t0;
     const uint32_t tmem = begin(ring, a.stages, a.cols);
+    pdl_release();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0 && lane == 0) {
         for (int kt = 0; kt < nk; ++kt) {
@@ -296,6 +305,7 @@ __global__ void __launch_bounds__(CONV_THREADS) k_wgrad(const __grid_constant__ 
         mma_commit(ring.done);
     }
     const bool ok = finish(ring);
+    pdl_wait();
     const int row = r0 + warp * 32 + lane;
     if (ok && nk > 0)
         for (int c0 = 0; c0 < a.nt && n0 + c0 < a.cout; c0 += 16) {
@@ -328,6 +338,7 @@ __global__ void __launch_bounds__(CONV_THREADS) k_wgrad_halo(const __grid_consta
     const int c0 = blockIdx.x * 32, n0 = blockIdx.z * a.nt;
     const int t0 = blockIdx.y * a.per, t1 = min(t0 + a.per, a.tiles), nk = t1 - t0;
     const uint32_t tmem = begin(ring, a.stages, a.cols);
+    pdl_release();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0 && lane == 0) {
         for (int kt = 0; kt < nk; ++kt) {
@@ -367,6 +378,7 @@ __global__ void __launch_bounds__(CONV_THREADS) k_wgrad_halo(const __grid_consta
         mma_commit(ring.done);
     }
     const bool ok = finish(ring);
+    pdl_wait();
     if (ok && nk > 0)
         for (int cc = 0; cc < 3 * a.nt; cc += 16) {
             const int dy = cc / a.nt, n = n0 + cc - dy * a.nt;
@@ -444,7 +456,7 @@ int launch_conv(cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, d
     const int rc = allow_smem(k_conv<KB, HALO>);
     if (rc != PAT_OK) return rc;
     count_launch();
-    k_conv<KB, HALO><<<grid, CONV_THREADS, smem, st>>>(ta, tb, a);
+    launch_pdl(k_conv<KB, HALO>, grid, dim3(CONV_THREADS), smem, st, true, ta, tb, a);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PAT_OK : cuda_fail(e, "k_conv");
 }
@@ -455,7 +467,7 @@ int launch_wgrad_halo(cudaStream_t st, const CUtensorMap& ta, const CUtensorMap&
     const int rc = allow_smem(k_wgrad_halo<CB>);
     if (rc != PAT_OK) return rc;
     count_launch();
-    k_wgrad_halo<CB><<<grid, CONV_THREADS, smem, st>>>(ta, tb, a);
+    launch_pdl(k_wgrad_halo<CB>, grid, dim3(CONV_THREADS), smem, st, true, ta, tb, a);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PAT_OK : cuda_fail(e, "k_wgrad_halo");
 }
@@ -466,7 +478,7 @@ int launch_wgrad(cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, 
     const int rc = allow_smem(k_wgrad<CA, CB>);
     if (rc != PAT_OK) return rc;
     count_launch();
-    k_wgrad<CA, CB><<<grid, CONV_THREADS, smem, st>>>(ta, tb, a);
+    launch_pdl(k_wgrad<CA, CB>, grid, dim3(CONV_THREADS), smem, st, true, ta, tb, a);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? PAT_OK : cuda_fail(e, "k_wgrad");
 }

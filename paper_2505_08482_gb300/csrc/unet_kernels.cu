@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "kfixed.cuh"
 #include "pat_internal.h"
 #include "unet.h"
 
@@ -195,6 +196,7 @@ union Bf8 {
 // rows of kp >= 9 C elements, the rest zero
 __global__ void k_im2col(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ col, int B, int H, int W,
                          int C, int ldc_in, int flip, int kp) {
+    pdl_wait_then_release();
     const int C8 = C / 8, K8 = kp / 8;
     const size_t total = size_t(B) * H * W * K8;
     GRID_STRIDE(i, total) {
@@ -235,6 +237,7 @@ __global__ void k_transpose(const __nv_bfloat16* __restrict__ in, __nv_bfloat16*
 // 2x2 max pooling (NHWC); idx records the argmax (0..3) for the backward
 __global__ void k_maxpool(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out,
                           unsigned char* __restrict__ idx, int B, int H, int W, int C) {
+    pdl_wait_then_release();
     const int Ho = H / 2, Wo = W / 2, C8 = C / 8;
     const size_t total = size_t(B) * Ho * Wo * C8;
     GRID_STRIDE(i, total) {
@@ -305,6 +308,7 @@ __global__ void k_enc_bwd(const __nv_bfloat16* __restrict__ dout, const unsigned
 // decoder input: cat = [nearest 2x upsampling of src (Cs channels) | skip (Ck channels)]
 __global__ void k_concat(const __nv_bfloat16* __restrict__ src, const __nv_bfloat16* __restrict__ skip,
                          __nv_bfloat16* __restrict__ cat, int B, int Hs, int Ws, int Cs, int Ck) {
+    pdl_wait_then_release();
     const int H = Hs * 2, W = Ws * 2, C8 = (Cs + Ck) / 8;
     const size_t total = size_t(B) * H * W * C8;
     GRID_STRIDE(i, total) {
@@ -365,6 +369,7 @@ __global__ void k_relu_bwd(__nv_bfloat16* __restrict__ g, const __nv_bfloat16* _
 constexpr int kBiasBlocks = 296;
 __global__ void __launch_bounds__(256) k_bias_grad(const __nv_bfloat16* __restrict__ g, float* __restrict__ part,
                                                    unsigned* __restrict__ done, float* __restrict__ db, size_t P, int C) {
+    pdl_wait_then_release();
     __shared__ float red[256][9];
     __shared__ bool last;
     const int c0 = blockIdx.y * 64, G = min(8, (C - c0) / 8);
@@ -592,7 +597,7 @@ int unet_transpose(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* out,
 }
 int unet_maxpool(cudaStream_t st, const __nv_bfloat16* in, __nv_bfloat16* out, unsigned char* idx, int B, int H, int W,
                  int C) {
-    k_maxpool<<<nblk(size_t(B) * H * W * C / 32), 256, 0, st>>>(in, out, idx, B, H, W, C);
+    launch_pdl(k_maxpool, nblk(size_t(B) * H * W * C / 32), dim3(256), 0, st, true, in, out, idx, B, H, W, C);
     LAUNCH_CHECK("k_maxpool");
     return PAT_OK;
 }
@@ -604,7 +609,8 @@ int unet_enc_bwd(cudaStream_t st, const __nv_bfloat16* dout, const unsigned char
 }
 int unet_concat(cudaStream_t st, const __nv_bfloat16* src, const __nv_bfloat16* skip, __nv_bfloat16* cat, int B, int Hs,
                 int Ws, int Cs, int Ck) {
-    k_concat<<<nblk(size_t(B) * Hs * Ws * 4 * (Cs + Ck) / 8), 256, 0, st>>>(src, skip, cat, B, Hs, Ws, Cs, Ck);
+    launch_pdl(k_concat, nblk(size_t(B) * Hs * Ws * 4 * (Cs + Ck) / 8), dim3(256), 0, st, true, src, skip, cat, B, Hs, Ws, Cs,
+               Ck);
     LAUNCH_CHECK("k_concat");
     return PAT_OK;
 }
@@ -623,7 +629,7 @@ int unet_bias_grad(cudaStream_t st, const __nv_bfloat16* g, float* db, float* pa
     // at least 16 pixels per thread: the last block's sum grows with the blocks
     const size_t group = 256 / std::min(8, C / 8);
     const unsigned nb = unsigned(std::max<size_t>(1, std::min<size_t>(kBiasBlocks, P / (16 * group))));
-    k_bias_grad<<<dim3(nb, (C + 63) / 64), 256, 0, st>>>(g, part, done, db, P, C);
+    launch_pdl(k_bias_grad, dim3(nb, (C + 63) / 64), dim3(256), 0, st, true, g, part, done, db, P, C);
     LAUNCH_CHECK("k_bias_grad");
     return PAT_OK;
 }

@@ -57,3 +57,32 @@ def test_gradients_refuse_a_pixel_count_that_is_no_multiple_of_8():
         net.gemm_path = path
         with pytest.raises(Bd.PatError):
             net.grads(x, torch.zeros((3, 20, 36), device="cuda"))
+
+
+def test_overlapped_launches_repeat():
+    """Forward passes and gradients repeat while their launches overlap, eagerly and from a captured graph: the outputs,
+    the loss and the bias gradients bit for bit, the weight gradients up to the order of their FP32 sums (1e-5: the
+    rounding of sums of a few thousand terms)."""
+    from paper_2505_08482_gb300.warmstart import UNet, init_params
+    B, in_ch, H, W = 8, 4, 64, 32
+    net = UNet(3, 32, in_ch, H, W, max_batch=B)
+    net.set_params(init_params(3, 32, in_ch))
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((B, in_ch, H, W), device="cuda", generator=gen)
+    t = torch.randn((B, H, W), device="cuda", generator=gen)
+    ref = net.forward(x).clone()
+    loss, g = net.grads(x, t)
+    g = g.clone()
+    head = g[-1].item()   # the last convolution's bias
+    for _ in range(10):
+        assert torch.equal(net.forward(x), ref)
+        l1, g1 = net.grads(x, t)
+        assert l1 == loss and g1[-1].item() == head and _rel(g1.cpu(), g.cpu()) <= 1e-5
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = net.forward(x)
+    for _ in range(10):
+        out.zero_()
+        graph.replay()
+        assert torch.equal(out, ref)
+    assert net.status() == 0
