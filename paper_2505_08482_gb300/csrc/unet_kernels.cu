@@ -457,7 +457,8 @@ __global__ void __launch_bounds__(256) k_head(const __nv_bfloat16* __restrict__ 
 
 // Loss L = mean (out - target)^2 and the backward of the final convolution in one pass over its input
 // y: d = bf16(2 (out - target) / n) per pixel, dy = [y > 0] bf16(d w), and per block the partial sums of
-// dW[c] = sum d y[c], db = sum d (part[b][C + 1]) and of the loss (lpart[b]).  Eight channels per thread.
+// dW[c] = sum d y[c], db = sum d (part[b][C + 1]) and of the loss (lpart[b]).  Eight channels per thread, so that
+// a block covers 2048 channels; blockIdx.y: the 2048 channels, of which the first also take db and the loss.
 constexpr int kHeadBlocks = 296;
 __global__ void __launch_bounds__(256) k_head_bwd(const float* __restrict__ out, const float* __restrict__ tgt,
                                                   const __nv_bfloat16* __restrict__ y,
@@ -465,8 +466,8 @@ __global__ void __launch_bounds__(256) k_head_bwd(const float* __restrict__ out,
                                                   float* __restrict__ part, double* __restrict__ lpart, size_t P, int C) {
     __shared__ float red[256][9];
     __shared__ double lred[256];
-    const int G = C / 8, R = 256 / G;   // C <= 2048
-    const int cg = threadIdx.x % G, pr = threadIdx.x / G;
+    const int g0 = blockIdx.y * 256, G = min(256, C / 8 - g0), R = 256 / G;
+    const int cg = g0 + threadIdx.x % G, pr = threadIdx.x / G;
     float wv[8], s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sb = 0.f;
     double ls = 0.0;
 #pragma unroll
@@ -494,19 +495,19 @@ __global__ void __launch_bounds__(256) k_head_bwd(const float* __restrict__ out,
     red[threadIdx.x][8] = sb;
     lred[threadIdx.x] = ls;
     __syncthreads();
-    for (int t = threadIdx.x; t <= C; t += 256) {
+    for (int t = threadIdx.x; t <= 8 * G; t += 256) {
         float v = 0.f;
-        if (t < C)
+        if (t < 8 * G)
             for (int r = 0; r < R; ++r) v += red[r * G + t / 8][t % 8];
         else
             for (int r = 0; r < R; ++r) v += red[r * G][8];
-        part[size_t(blockIdx.x) * (C + 1) + t] = v;
+        if (t < 8 * G || g0 == 0) part[size_t(blockIdx.x) * (C + 1) + (t < 8 * G ? 8 * g0 + t : C)] = v;
     }
     for (int k = 128; k > 0; k >>= 1) {
         __syncthreads();
         if (threadIdx.x < k) lred[threadIdx.x] += lred[threadIdx.x + k];
     }
-    if (threadIdx.x == 0) lpart[blockIdx.x] = lred[0];
+    if (threadIdx.x == 0 && g0 == 0) lpart[blockIdx.x] = lred[0];
 }
 __global__ void k_head_sum(const float* __restrict__ part, const double* __restrict__ lpart, int nblk,
                            float* __restrict__ dw, float* __restrict__ db, double* __restrict__ loss, double scale, int C) {
@@ -643,7 +644,7 @@ int unet_head(cudaStream_t st, const __nv_bfloat16* y, const __nv_bfloat16* w, c
 }
 int unet_head_bwd(cudaStream_t st, const float* out, const float* tgt, const __nv_bfloat16* y, const __nv_bfloat16* w,
                   __nv_bfloat16* dy, float* part, double* lpart, float* dw, float* db, double* loss, size_t P, int C) {
-    k_head_bwd<<<kHeadBlocks, 256, 0, st>>>(out, tgt, y, w, dy, part, lpart, P, C);
+    k_head_bwd<<<dim3(kHeadBlocks, (C / 8 + 255) / 256), 256, 0, st>>>(out, tgt, y, w, dy, part, lpart, P, C);
     LAUNCH_CHECK("k_head_bwd");
     k_head_sum<<<C + 2, 32, 0, st>>>(part, lpart, kHeadBlocks, dw, db, loss, 1.0 / double(P), C);
     LAUNCH_CHECK("k_head_sum");
