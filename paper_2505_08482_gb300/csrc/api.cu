@@ -189,8 +189,7 @@ int reverse_sweep(pat_plan_s* p, const float* p0, const float* r, float* grad_p0
         return launch_reduce_cbar(L, w, grad_c);
     }
     RC(launch_row_adj_final1(L, w, have_q ? 0 : 1, r, grad_p0));
-    const float s0 = float(-0.5 * p->g.dt / p->g.rho0 / (double(p->ng) * p->ng));
-    RC(launch_col(L, w.A2, w.B2, 2, 1, s0));
+    RC(launch_col(L, w.A2, w.B2, 2, 1, -0.5f * sd));   // transpose of the initial half step
     RC(launch_row_adj_final2(L, w, p0, grad_p0));
     RC(launch_reduce_cbar(L, w, grad_c));
     return PAT_OK;
