@@ -200,7 +200,8 @@ int pat_plan_set_graphs(pat_plan plan, int enable);
  * workspace (d_ws NULL: a temporary one is allocated and freed on the
  * stream).  The workspace contents are overwritten.  h_ms: host array of
  * pat_plan_variants(plan)+1 entries (may be NULL) receiving, for variants
- * -1, 0, ..., the ms per gradient evaluation or per forward step.
+ * -1, 0, ..., the ms per gradient evaluation or per forward step (infinity for
+ * the split-axis step in a workspace that holds the four-pass step only).
  * Synchronises the stream; with no fixed-size variant it selects -1. */
 int pat_plan_autotune(pat_plan plan, void* d_ws, size_t ws_bytes, double* h_ms, void* stream);
 
@@ -211,16 +212,25 @@ int pat_pml_auto(int n, int min_pml);
 
 /* Workspace sizes in bytes (caller allocates, 256-byte aligned device
  * memory).  PAT_WS_FORWARD suffices for pat_forward; PAT_WS_GRADIENT holds
- * the checkpoints and the adjoint state as well. */
+ * the checkpoints and the adjoint state as well.  Where the plan has the
+ * split-axis step (pat_plan_set_variant), these sizes hold its state, which is
+ * larger than the four-pass step's.  A workspace that holds the four-pass step
+ * only is accepted by every call that takes a workspace, and the call then
+ * runs the four-pass step (variant 0: its form with mixed factorisations; else the generic
+ * passes): with F = 4 K Ng^2 and S = 8 K Ng P bytes (P: Ng / 2 + 1 rounded up to
+ * a multiple of 4) its state is 4 F + 2 S, in PAT_WS_GRADIENT twice, instead of
+ * 24 K Ng (Ng + 2) + 2 F (each array rounded up to 256 bytes).  Such a gradient
+ * workspace has its checkpoints where the larger one has them. */
 #define PAT_WS_FORWARD 0
 #define PAT_WS_GRADIENT 1
 size_t pat_workspace_bytes(pat_plan plan, int kind);
 
 /* Forward operator (Eq. ObservationModel without noise): d_y[k][n][m] =
  * S p_k^n for the K initial pressures d_p0 [K][N][N] and the speed of sound
- * d_c [N][N].  d_y [K][nt][m] is overwritten.  If ws_bytes >=
- * pat_workspace_bytes(plan, PAT_WS_GRADIENT) the checkpoints needed by a
- * following pat_vjp with the same c and p0 are kept in d_ws. */
+ * d_c [N][N].  d_y [K][nt][m] is overwritten.  If d_ws is a gradient
+ * workspace (ws_bytes >= pat_workspace_bytes(plan, PAT_WS_GRADIENT), or the
+ * four-pass step's size of it) the checkpoints needed by a following pat_vjp
+ * with the same c and p0 are kept in d_ws. */
 int pat_forward(pat_plan plan, const float* d_c, const float* d_p0, float* d_y,
                 void* d_ws, size_t ws_bytes, void* stream);
 
@@ -233,9 +243,9 @@ int pat_forward(pat_plan plan, const float* d_c, const float* d_p0, float* d_y,
  * pat_forward.  Same arguments and results as pat_forward without the
  * workspace: the scratch is a static device array of
  * PAT_NOALLOC_SCRATCH_BYTES (16 MiB) that every GPU loading the library
- * holds until exit.  Plans whose forward workspace
- * (pat_workspace_bytes(plan, PAT_WS_FORWARD)) exceeds it are rejected with
- * PAT_EINVAL and a message.  The plan's device must be current.  The array's
+ * holds until exit.  Plans whose forward workspace (that of the four-pass step,
+ * which such a call then runs) exceeds it are rejected with PAT_EINVAL and a
+ * message.  The plan's device must be current.  The array's
  * device address is looked up in the current context on every call (after a
  * cudaDeviceReset it may move); the first call in a context loads the
  * library's device code (set-up), so make it before any stream capture.  All

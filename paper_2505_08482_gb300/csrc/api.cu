@@ -45,6 +45,9 @@ int step(const Launch& L, const Ws& w, int n, float* y, float* hist, int hist_sl
     return PAT_OK;
 }
 
+// the split-axis passes of the plan where the workspace holds their larger state, else the four-pass step
+const SplitOps* split_of(const pat_plan_s* p, const Ws& w) { return w.split_fits ? p->split : nullptr; }
+
 size_t state_bytes(const pat_plan_s* p) { return 4 * size_t(p->K) * p->ng * p->ng * sizeof(float); }
 
 // forward steps n0 .. n1-1; p^{n+1} into hist slot n+1-hbase when hist and n+1 >= hbase
@@ -60,9 +63,9 @@ int run_steps(const Launch& L, const Ws& w, int n0, int n1, float* y, float* his
 }  // namespace
 
 int pat::forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y, const Ws& w, bool keep,
-                       cudaStream_t st, bool allow_split) {
+                       cudaStream_t st) {
     NvtxRange nv("pat forward sweep");
-    Launch L{p, st, true, false, allow_split ? p->split : nullptr};
+    Launch L{p, st, true, false, split_of(p, w)};
     RC(launch_medium(L, c, w.cg));
     PAT_CUDA(cudaMemsetAsync(y, 0, size_t(p->K) * p->nt * p->m * sizeof(float), st));
     PAT_CUDA(cudaMemsetAsync(w.flag + 1, 0, sizeof(int), st));   // bounded-wait status of this call
@@ -101,7 +104,7 @@ namespace {
 
 // recompute segment j's pressure history into its buffer (on stream st)
 int recompute(pat_plan_s* p, const float* p0, const Ws& w, int j, cudaStream_t st) {
-    Launch L{p, st, false, true, p->split};
+    Launch L{p, st, false, true, split_of(p, w)};
     const size_t f = size_t(p->K) * p->ng * p->ng;
     const int n0 = j * p->s_eff;
     const int n1 = std::min(n0 + p->s_eff, p->nt) - 1;
@@ -143,7 +146,7 @@ int run_adj(const Launch& L, const Ws& w, const float* r, int n_hi, int n_lo, bo
 int reverse_sweep(pat_plan_s* p, const float* p0, const float* r, float* grad_p0, float* grad_c, const Ws& w,
                   bool hist_last_valid, cudaStream_t st) {
     NvtxRange nv("pat reverse sweep");
-    Launch L{p, st, false, false, p->split};
+    Launch L{p, st, false, false, split_of(p, w)};
     const size_t f = size_t(p->K) * p->ng * p->ng;
     if (L.split) {
         const size_t lines = 2 * size_t(p->K) * p->hc * p->ng * sizeof(float2);
@@ -239,7 +242,7 @@ int with_graph(pat_plan_s* p, int kind, const std::array<const void*, 10>& key, 
 int check_ws(const pat_plan_s* p, const void* ws, size_t bytes, bool grad) {
     if (!ws) { set_error("workspace is NULL"); return PAT_EINVAL; }
     if (reinterpret_cast<uintptr_t>(ws) % 256 != 0) { set_error("workspace must be 256-byte aligned"); return PAT_EINVAL; }
-    const size_t need = grad ? p->ws_grad : p->ws_fwd;
+    const size_t need = grad ? p->ws_grad_passes : p->ws_fwd_passes;
     if (bytes < need) {
         set_error("workspace too small: %zu < %zu bytes", bytes, need);
         return PAT_ENOMEM;
@@ -252,7 +255,7 @@ int check_ws(const pat_plan_s* p, const void* ws, size_t bytes, bool grad) {
 int pat::objective(pat_plan_s* p, const float* c, const float* p0, const float* ymeas, const float* wts,
                    double* J_dev, void* ws, size_t ws_bytes, cudaStream_t st) {
     RC(check_ws(p, ws, ws_bytes, true));
-    Ws w = resolve(p, ws, true);
+    Ws w = resolve(p, ws, ws_bytes, true);
     RC(with_graph(p, 0, {c, p0, ymeas, wts, J_dev, ws}, ws_bytes, st, [&]() -> int {
         RC(forward_sweep(p, c, p0, w.ypred, w, false, st));
         Launch L{p, st};
@@ -268,8 +271,8 @@ extern "C" int pat_forward(pat_plan p, const float* c, const float* p0, float* y
                            void* stream) {
     if (!p || !c || !p0 || !y) { set_error("pat_forward: null argument"); return PAT_EINVAL; }
     RC(check_ws(p, ws, ws_bytes, false));
-    const bool keep = ws_bytes >= p->ws_grad;
-    Ws w = resolve(p, ws, keep);
+    const bool keep = ws_bytes >= p->ws_grad_passes;
+    Ws w = resolve(p, ws, ws_bytes, keep);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     RC(with_graph(p, keep ? 2 : 1, {c, p0, y, ws}, ws_bytes, st,
                   [&]() -> int { return forward_sweep(p, c, p0, y, w, keep, st); }));
@@ -285,7 +288,7 @@ extern "C" int pat_adjoint_grad(pat_plan p, const float* c, const float* p0, con
         return PAT_EINVAL;
     }
     RC(check_ws(p, ws, ws_bytes, true));
-    Ws w = resolve(p, ws, true);
+    Ws w = resolve(p, ws, ws_bytes, true);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     float* yp = y_pred ? y_pred : w.ypred;
     RC(with_graph(p, 3, {c, p0, y_meas, wts, grad_p0, grad_c, J, y_pred, ws}, ws_bytes, st, [&]() -> int {
@@ -303,7 +306,7 @@ extern "C" int pat_vjp(pat_plan p, const float* c, const float* p0, const float*
                        void* ws, size_t ws_bytes, void* stream) {
     if (!p || !c || !p0 || !ybar || !grad_p0 || !grad_c) { set_error("pat_vjp: null argument"); return PAT_EINVAL; }
     RC(check_ws(p, ws, ws_bytes, true));
-    Ws w = resolve(p, ws, true);
+    Ws w = resolve(p, ws, ws_bytes, true);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     Launch L{p, st};
     PAT_CUDA(cudaMemsetAsync(w.flag + 1, 0, sizeof(int), st));   // bounded-wait status of this call
@@ -328,7 +331,7 @@ extern "C" int pat_plan_autotune(pat_plan p, void* ws, size_t ws_bytes, double* 
         ws = own;
         ws_bytes = p->ws_fwd;
     }
-    const bool grad = ws_bytes >= p->ws_grad;
+    const bool grad = ws_bytes >= p->ws_grad_passes;
     int rc = check_ws(p, ws, ws_bytes, grad);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     float* tmp = nullptr;   // gradient mode: c, p0, dJ/dp0, dJ/dc
@@ -338,7 +341,7 @@ extern "C" int pat_plan_autotune(pat_plan p, void* ws, size_t ws_bytes, double* 
     int bestv = -1;
     if (rc == PAT_OK) {
         // zero state, spectra and residual; the timed passes then run on finite values
-        if (cudaMemsetAsync(ws, 0, grad ? p->ws_grad : p->ws_fwd, st) != cudaSuccess ||
+        if (cudaMemsetAsync(ws, 0, std::min(ws_bytes, grad ? p->ws_grad : p->ws_fwd), st) != cudaSuccess ||
             cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
             rc = cuda_fail(cudaGetLastError(), "pat_plan_autotune");
     }
@@ -348,7 +351,7 @@ extern "C" int pat_plan_autotune(pat_plan p, void* ws, size_t ws_bytes, double* 
             rc = cuda_fail(cudaGetLastError(), "pat_plan_autotune buffers");
         if (rc == PAT_OK) rc = vfill(st, tmp, float(p->g.c_ref), size_t(p->ninst) * nn);
     }
-    Ws w = resolve(p, ws, grad);
+    Ws w = resolve(p, ws, ws_bytes, grad);
     Launch L{p, st, true};   // forward-step timing mirrors the forward sweep
     float* c = tmp;
     float* p0 = tmp ? tmp + size_t(p->ninst) * nn : nullptr;
@@ -358,6 +361,10 @@ extern "C" int pat_plan_autotune(pat_plan p, void* ws, size_t ws_bytes, double* 
     for (int v = -1; v < nv && rc == PAT_OK; ++v) {
         rc = select_variant(p, v);
         if (rc != PAT_OK) break;
+        if (p->split && !w.split_fits) {   // the calls with this workspace would run another form
+            if (h_ms) h_ms[v + 1] = HUGE_VAL;
+            continue;
+        }
         L.split = p->split;
         rc = run_steps(L, w, 1, 4, nullptr, nullptr, 0);   // first launches of the variant's kernels
         if (rc != PAT_OK) break;

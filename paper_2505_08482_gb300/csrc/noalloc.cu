@@ -67,10 +67,9 @@ extern "C" int pat_forward_noalloc(pat_plan p, const float* c, const float* p0, 
     if (rc != PAT_OK) return rc;
     // the forward sweep writes every scratch region it reads before reading it,
     // so nothing left by an earlier call needs clearing
-    pat::Ws w = pat::resolve(p, scratch, false);
-    // the split-axis passes where their larger state fits the array too, else the four-pass step
-    rc = pat::forward_sweep(p, c, p0, y, w, false, static_cast<cudaStream_t>(stream),
-                            p->ws_fwd <= size_t(PAT_NOALLOC_SCRATCH_BYTES));
+    // (the split-axis passes where their larger state fits the array too, else the four-pass step)
+    pat::Ws w = pat::resolve(p, scratch, PAT_NOALLOC_SCRATCH_BYTES, false);
+    rc = pat::forward_sweep(p, c, p0, y, w, false, static_cast<cudaStream_t>(stream));
     if (rc != PAT_OK) return rc;
     p->hist_valid_ws = nullptr;
     return PAT_OK;

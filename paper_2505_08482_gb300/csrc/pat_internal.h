@@ -64,6 +64,7 @@ struct Ws {
     float2* A; float2* B;                         // spectra [K][ng][hc]
     double* J; double* part; int* flag;           // objective per instance, partial sums [K][32], flag
     int* queue;                                   // persistent sweep: tickets, abort flag, done per data set
+    bool split_fits;                              // the workspace holds the split-axis passes' state too
     // the split-axis passes' view of the same memory: lines [2][K][hc][ng] of u, rho and the pressure,
     // real rho_x, rho_y [2][K][ng][ng]; the adjoint's below
     float2* lu; float2* lr; float2* la; float* re;
@@ -102,11 +103,12 @@ struct pat_plan_s {
     pat::Tables t;
     int nent;
     size_t ws_fwd, ws_grad;
-    size_t ws_fwd_passes;   // forward workspace of the four-pass step alone
-    // layout offsets (bytes)
-    size_t o_state, o_cg, o_A, o_B, o_J, o_part, o_flag, o_queue;
-    size_t o_ckpt, o_hist, o_adj, o_A2, o_B2, o_cbar, o_resid, o_ypred;
-    size_t o_lu, o_lr, o_la, o_re, o_lub, o_lrb, o_la2, o_re2;   // split-axis views
+    size_t ws_fwd_passes, ws_grad_passes;   // workspaces of the four-pass step alone
+    // layout offsets (bytes): in a workspace, and within the state of a step
+    size_t o_state, o_state_grad, o_cg, o_J, o_part, o_flag, o_queue;
+    size_t o_ckpt, o_hist, o_cbar, o_resid, o_ypred;
+    size_t s_A, s_B, s_passes;          // four-pass step: spectra, size
+    size_t s_lr, s_la, s_re, s_most;    // split-axis passes: lines of rho and the pressure, real fields; larger size
     // host bookkeeping: the workspace whose history holds the last segment
     const void* hist_valid_ws;
     int device;
@@ -133,7 +135,7 @@ struct pat_plan_s {
 
 namespace pat {
 
-Ws resolve(const pat_plan_s* p, void* base, bool grad);
+Ws resolve(const pat_plan_s* p, void* base, size_t bytes, bool grad);
 
 // pressure history buffer of segment j (segments alternate between two buffers)
 inline float* hist_of(const pat_plan_s* p, const Ws& w, int j) {
@@ -218,9 +220,8 @@ int split_configure(const SplitOps* ops);
 float scale_g(const pat_plan_s* p);
 float scale_d(const pat_plan_s* p);
 // Forward sweep into y [K][nt][m] with workspace regions w (checkpoints kept if keep).
-// allow_split = false: the four-pass step (a workspace too small for the split-axis passes).
 int forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y, const Ws& w, bool keep,
-                  cudaStream_t st, bool allow_split = true);
+                  cudaStream_t st);
 // used by the reconstruction driver:
 // J only (forward sweep + residual) into *J_dev; workspace of PAT_WS_GRADIENT size.
 int objective(pat_plan_s* p, const float* c, const float* p0, const float* ymeas, const float* wts, double* J_dev,

@@ -76,89 +76,84 @@ static double pml_factor(const pat_grid& g, int P, double s) {
     return std::exp(-0.5 * alpha * g.dt);
 }
 
-Ws resolve(const pat_plan_s* p, void* base, bool grad) {
+Ws resolve(const pat_plan_s* p, void* base, size_t bytes, bool grad) {
     char* b = static_cast<char*>(base);
     Ws w{};
+    w.split_fits = bytes >= (grad ? p->ws_grad : p->ws_fwd);
     const size_t f = size_t(p->K) * p->ng * p->ng;
-    float* st = reinterpret_cast<float*>(b + p->o_state);
-    w.ux = st;
-    w.uy = st + f;
-    w.rx = st + 2 * f;
-    w.ry = st + 3 * f;
     w.cg = reinterpret_cast<float*>(b + p->o_cg);
-    w.A = reinterpret_cast<float2*>(b + p->o_A);
-    w.B = reinterpret_cast<float2*>(b + p->o_B);
     w.J = reinterpret_cast<double*>(b + p->o_J);
     w.part = reinterpret_cast<double*>(b + p->o_part);
     w.flag = reinterpret_cast<int*>(b + p->o_flag);
     w.queue = reinterpret_cast<int*>(b + p->o_queue);
-    w.lu = reinterpret_cast<float2*>(b + p->o_lu);
-    w.lr = reinterpret_cast<float2*>(b + p->o_lr);
-    w.la = reinterpret_cast<float2*>(b + p->o_la);
-    w.re = reinterpret_cast<float*>(b + p->o_re);
+    auto four = [f](char* at, float* (&v)[4]) {
+        for (int i = 0; i < 4; ++i) v[i] = reinterpret_cast<float*>(at) + i * f;
+    };
+    char* st = b + (grad ? p->o_state_grad : p->o_state);
+    float* v[4];
+    four(st, v);
+    w.ux = v[0]; w.uy = v[1]; w.rx = v[2]; w.ry = v[3];
+    w.A = reinterpret_cast<float2*>(st + p->s_A);
+    w.B = reinterpret_cast<float2*>(st + p->s_B);
+    w.lu = reinterpret_cast<float2*>(st);
+    w.lr = reinterpret_cast<float2*>(st + p->s_lr);
+    w.la = reinterpret_cast<float2*>(st + p->s_la);
+    w.re = reinterpret_cast<float*>(st + p->s_re);
     if (grad) {
-        w.lub = reinterpret_cast<float2*>(b + p->o_lub);
-        w.lrb = reinterpret_cast<float2*>(b + p->o_lrb);
-        w.la2 = reinterpret_cast<float2*>(b + p->o_la2);
-        w.re2 = reinterpret_cast<float*>(b + p->o_re2);
         w.ckpt = reinterpret_cast<float*>(b + p->o_ckpt);
         w.hist = reinterpret_cast<float*>(b + p->o_hist);
-        float* ad = reinterpret_cast<float*>(b + p->o_adj);
-        w.ubx = ad;
-        w.uby = ad + f;
-        w.rbx = ad + 2 * f;
-        w.rby = ad + 3 * f;
-        w.A2 = reinterpret_cast<float2*>(b + p->o_A2);
-        w.B2 = reinterpret_cast<float2*>(b + p->o_B2);
         w.cbar = reinterpret_cast<float*>(b + p->o_cbar);
         w.resid = reinterpret_cast<float*>(b + p->o_resid);
         w.ypred = reinterpret_cast<float*>(b + p->o_ypred);
+        // the adjoint state: the same regions again behind the forward state
+        char* ad = st + (w.split_fits ? p->s_most : p->s_passes);
+        four(ad, v);
+        w.ubx = v[0]; w.uby = v[1]; w.rbx = v[2]; w.rby = v[3];
+        w.A2 = reinterpret_cast<float2*>(ad + p->s_A);
+        w.B2 = reinterpret_cast<float2*>(ad + p->s_B);
+        w.lub = reinterpret_cast<float2*>(ad);
+        w.lrb = reinterpret_cast<float2*>(ad + p->s_lr);
+        w.la2 = reinterpret_cast<float2*>(ad + p->s_la);
+        w.re2 = reinterpret_cast<float*>(ad + p->s_re);
     }
     return w;
 }
 
-// The four-pass step and the split-axis passes lay their state over the same memory (a plan runs one
-// of them at a time; checkpoints and the pressure history are real fields in both).
+// What outlives a call (checkpoints, history, status) comes first; the state of a step follows, the four-pass step's
+// and the split-axis passes' over the same memory (a call runs one of them; checkpoints and the pressure history are
+// real fields in both).  A workspace that holds the four-pass step only is laid out alike up to that state, so that
+// calls with workspaces of either size share checkpoints.
 static void layout(pat_plan_s* p) {
     const size_t f = size_t(p->K) * p->ng * p->ng * sizeof(float);
     const size_t spec = size_t(p->K) * p->ng * p->hp * sizeof(float2);
     const size_t lines = 2 * size_t(p->K) * p->hc * p->ng * sizeof(float2);
-    const bool split = split_ops_for(p->ng) != nullptr;
+    size_t q = align256(4 * f);   // four-pass: state, two spectra
+    p->s_A = q; q = align256(q + spec);
+    p->s_B = q; q = align256(q + spec);
+    p->s_passes = p->s_most = q;
+    q = align256(lines);          // split-axis: lines of u, rho and the pressure, two real fields
+    p->s_lr = q; q = align256(q + lines);
+    p->s_la = q; q = align256(q + lines);
+    p->s_re = q; q = align256(q + 2 * f);
+    if (split_ops_for(p->ng)) p->s_most = std::max(p->s_passes, q);
     size_t o = 0;
     p->o_cg = o; o = align256(o + size_t(p->ninst) * p->ng * p->ng * sizeof(float));
     p->o_J = o; o = align256(o + size_t(p->ninst) * sizeof(double));
     p->o_part = o; o = align256(o + size_t(p->K) * kResidBlocks * sizeof(double));
     p->o_flag = o; o = align256(o + 4 * sizeof(int));
     p->o_queue = o; o = align256(o + (size_t(p->K) + 2) * sizeof(int));
-    const size_t fwd = o;
-    p->o_state = o; o = align256(o + 4 * f);
-    p->o_A = o; o = align256(o + spec);
-    p->o_B = o; o = align256(o + spec);
-    p->ws_fwd_passes = o;
-    size_t q = fwd;
-    p->o_lu = q; q = align256(q + lines);
-    p->o_lr = q; q = align256(q + lines);
-    p->o_la = q; q = align256(q + lines);
-    p->o_re = q; q = align256(q + 2 * f);
-    if (split) o = std::max(o, q);
-    p->ws_fwd = o;
+    p->o_state = o;
+    p->ws_fwd_passes = o + p->s_passes;
+    p->ws_fwd = o + p->s_most;
     p->o_ckpt = o; o = align256(o + size_t(std::max(p->nseg - 1, 0)) * 4 * f);
     p->o_hist = o; o = align256(o + size_t(p->nseg > 1 ? 2 : 1) * p->K * p->s_eff * p->ng * p->ng * sizeof(float));
-    const size_t adj = o;
-    p->o_adj = o; o = align256(o + 4 * f);
-    p->o_A2 = o; o = align256(o + spec);
-    p->o_B2 = o; o = align256(o + spec);
-    q = adj;
-    p->o_lub = q; q = align256(q + lines);
-    p->o_lrb = q; q = align256(q + lines);
-    p->o_la2 = q; q = align256(q + lines);
-    p->o_re2 = q; q = align256(q + 2 * f);
-    if (split) o = std::max(o, q);
     p->o_cbar = o; o = align256(o + size_t(p->K) * p->n * p->n * sizeof(float));
     const size_t tr = size_t(p->K) * p->nt * p->m * sizeof(float);
     p->o_resid = o; o = align256(o + tr);
     p->o_ypred = o; o = align256(o + tr);
-    p->ws_grad = o;
+    p->o_state_grad = o;
+    p->ws_grad_passes = o + 2 * p->s_passes;
+    p->ws_grad = o + 2 * p->s_most;
 }
 
 }  // namespace pat
