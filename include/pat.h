@@ -134,13 +134,18 @@ int pat_plan_ng(pat_plan plan);
  *      register FFT (60 threads per column), 4 / 8 and 2 / 4 columns per CTA;
  *   9  (300) as 5 with 4-column tiles in the forward sweep's column passes;
  *   10 (300) as 5 with the column passes of 7 (108-240).
- * Every side also has the generic shared-memory Stockham passes (variant
- * -1); on sides without variants -1 is the split-axis step where it is
- * compiled (72, 80, 90, 96, 100, 120, 128, 150, 160, 192, 216, 250, 256, 270,
- * 288, 320, 324, 360, 384, 400).  All variants compute the same scheme.  A new plan uses variant 0
- * when it exists, else -1.  pat_plan_variants returns the number of
- * fixed-size variants; pat_plan_set_variant selects one (PAT_EINVAL if it
- * does not exist); pat_plan_variant returns the current one. */
+ * Every side also has the generic shared-memory Stockham passes: variant -1
+ * on sides with variants and on sides without the split-axis step.  On the
+ * sides without variants for which the split-axis step is compiled (72, 80,
+ * 90, 96, 100, 120, 128, 150, 160, 192, 216, 250, 256, 270, 288, 320, 324, 360,
+ * 384, 400) variant -1 is that step, and PAT_VARIANT_GENERIC selects (and
+ * pat_plan_variant then reports) the generic passes; on all other sides
+ * PAT_VARIANT_GENERIC is -1.  All variants compute the same scheme.  A new plan
+ * uses variant 0 when it exists, else -1.  pat_plan_variants returns the number
+ * of fixed-size variants; pat_plan_set_variant selects one (PAT_EINVAL if it
+ * does not exist; negative values other than PAT_VARIANT_GENERIC: -1);
+ * pat_plan_variant returns the current one (-2 for a NULL plan). */
+#define PAT_VARIANT_GENERIC (-3)
 int pat_plan_variants(pat_plan plan);
 int pat_plan_set_variant(pat_plan plan, int variant);
 int pat_plan_variant(pat_plan plan);
@@ -202,7 +207,8 @@ int pat_plan_set_graphs(pat_plan plan, int enable);
  * pat_plan_variants(plan)+1 entries (may be NULL) receiving, for variants
  * -1, 0, ..., the ms per gradient evaluation or per forward step (infinity for
  * the split-axis step in a workspace that holds the four-pass step only).
- * Synchronises the stream; with no fixed-size variant it selects -1. */
+ * Synchronises the stream; with no fixed-size variant it selects -1 (also
+ * when PAT_VARIANT_GENERIC was selected, whose passes it does not time). */
 int pat_plan_autotune(pat_plan plan, void* d_ws, size_t ws_bytes, double* h_ms, void* stream);
 
 /* Smallest PML width >= min_pml for which n + 2 P satisfies the grid rules

@@ -31,6 +31,7 @@ PAT_K_TO_LINES = 9
 PAT_K_TO_REAL = 10
 KERNEL_CLASSES = {1: "k_row_rho", 2: "k_row_u", 3: "k_col(grad)", 4: "k_col(pair)", 5: "k_col(sum)",
                   6: "k_row_adj_rho", 7: "k_row_adj_u", 8: "ks_lines", 9: "ks_to_lines", 10: "ks_to_real"}
+PAT_VARIANT_GENERIC = -3
 PAT_WS_FORWARD = 0
 PAT_NOALLOC_SCRATCH_BYTES = 16 * 1024 * 1024
 PAT_WS_GRADIENT = 1

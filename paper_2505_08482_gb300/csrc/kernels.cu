@@ -579,10 +579,12 @@ int configure_kernels(pat_plan_s* p) {
 }
 
 int select_variant(pat_plan_s* p, int variant) {
-    // the split-axis passes are variant 0 of the sides that have variants and the only form of the
-    // others (which report the generic variant -1)
+    // the split-axis passes are variant 0 of the sides that have variants and variant -1 of the others, whose
+    // generic passes are PAT_VARIANT_GENERIC
     const SplitOps* sp = split_ops_for(p->ng);
-    if (variant > 0 || (variant < 0 && fixed_variants(p->ng) > 0)) sp = nullptr;
+    const bool generic = variant < 0 && (!sp || variant == PAT_VARIANT_GENERIC || fixed_variants(p->ng) > 0);
+    const int name = generic && sp && fixed_variants(p->ng) == 0 ? PAT_VARIANT_GENERIC : -1;
+    if (variant > 0 || generic) sp = nullptr;
     if (sp) {
         const int rc = split_configure(sp);
         if (rc != PAT_OK) return rc;
@@ -590,7 +592,7 @@ int select_variant(pat_plan_s* p, int variant) {
     if (variant < 0) {
         p->fast = nullptr;
         p->split = sp;
-        p->variant = -1;
+        p->variant = name;
         return PAT_OK;
     }
     const FixedOps* f = fixed_ops_for(p->ng, variant);

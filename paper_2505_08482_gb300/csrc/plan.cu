@@ -186,7 +186,7 @@ extern "C" int pat_plan_set_variant(pat_plan plan, int variant) {
         set_error("pat_plan_set_variant: grid side %d has %d fixed-size variants", plan->ng, fixed_variants(plan->ng));
         return PAT_EINVAL;
     }
-    return select_variant(plan, variant < 0 ? -1 : variant);
+    return select_variant(plan, variant < 0 && variant != PAT_VARIANT_GENERIC ? -1 : variant);
 }
 
 extern "C" int pat_plan_variant(pat_plan plan) { return plan ? plan->variant : -2; }

@@ -114,11 +114,13 @@ class Plan:
 
     @property
     def variants(self) -> int:
-        """Number of fixed-size kernel variants for this grid side (0: generic only)."""
+        """Number of fixed-size kernel variants for this grid side (0: none; see ``variant``)."""
         return int(B.lib().pat_plan_variants(self._h))
 
     @property
     def variant(self) -> int:
+        """Kernel variant in use (pat_plan_set_variant): 0 .. variants - 1, -1, or PAT_VARIANT_GENERIC for the
+        generic passes of a side whose variant -1 is the split-axis step."""
         return int(B.lib().pat_plan_variant(self._h))
 
     @variant.setter
