@@ -112,8 +112,8 @@ int pat_plan_shape(pat_plan plan, int* ninst, int* K);
 int pat_plan_ng(pat_plan plan);
 
 /* Kernel variants of a plan.  Grid sides with a compiled two-level FFT
- * (108, 144, 180, 200, 240, 300 = N1 x N2) have fixed-size variants (eight
- * for 108-240, eleven for 300).  Variant 0, the default, is the split-axis
+ * (108, 144, 180, 200, 240, 300 = N1 x N2) have fixed-size variants (nine
+ * for 108-240, twelve for 300).  Variant 0, the default, is the split-axis
  * step, three launches per time step on the lines of the half spectra along
  * each axis; the others are the four-pass step, one launch per pass:
  *   1  all passes N1 x N2, 4 rows / 4 columns per CTA;
@@ -133,7 +133,8 @@ int pat_plan_ng(pat_plan plan);
  *   7, 8 (300) as 5 with the column passes on a three-level 5 x 10 x 6
  *      register FFT (60 threads per column), 4 / 8 and 2 / 4 columns per CTA;
  *   9  (300) as 5 with 4-column tiles in the forward sweep's column passes;
- *   10 (300) as 5 with the column passes of 7 (108-240).
+ *   10 (300) as 5 with the column passes of 7 (108-240);
+ *   8 (108-240), 11 (300) as 5 with 4 rows per CTA in the row passes.
  * Every side also has the generic shared-memory Stockham passes: variant -1
  * on sides with variants and on sides without the split-axis step.  On the
  * sides without variants for which the split-axis step is compiled (72, 80,
@@ -222,7 +223,7 @@ int pat_pml_auto(int n, int min_pml);
  * split-axis step (pat_plan_set_variant), these sizes hold its state, which is
  * larger than the four-pass step's.  A workspace that holds the four-pass step
  * only is accepted by every call that takes a workspace, and the call then
- * runs the four-pass step (variant 0: its form with mixed factorisations; else the generic
+ * runs the four-pass step (variant 0: the plan's last variant; else the generic
  * passes): with F = 4 K Ng^2 and S = 8 K Ng P bytes (P: Ng / 2 + 1 rounded up to
  * a multiple of 4) its state is 4 F + 2 S, in PAT_WS_GRADIENT twice, instead of
  * 24 K Ng (Ng + 2) + 2 F (each array rounded up to 256 bytes).  Such a gradient

@@ -19,7 +19,7 @@ const ClusterOps* cluster_ops_300();
 
 const ClusterOps* cluster_ops_for(int ng) { return ng == 300 ? cluster_ops_300() : nullptr; }
 
-const FixedOps* fixed_ops_for(int ng, int v) {
+static const FixedOps* entry(int ng, int v) {
     switch (ng) {
         case 108: return fixed_ops_108(v);
         case 144: return fixed_ops_144(v);
@@ -29,6 +29,13 @@ const FixedOps* fixed_ops_for(int ng, int v) {
         case 300: return fixed_ops_300(v);
         default: return nullptr;
     }
+}
+
+// Variant 0 of a plan is the split-axis step, beside which entry 0, the mixed four-pass form, serves what is not stepped
+// by it; as a variant of its own that form is the last one.
+const FixedOps* fixed_ops_for(int ng, int v) {
+    if (const FixedOps* f = entry(ng, v)) return f;
+    return v > 0 && entry(ng, v - 1) ? entry(ng, 0) : nullptr;
 }
 
 const SweepOps* sweep_ops_for(int ng) {

@@ -1,4 +1,6 @@
-// Fixed-size passes for the grid side Ng = 180 = 12 x 15.  Variants: 0 column and velocity
+// Fixed-size passes of the four-pass step for the grid side Ng = 180 = 12 x 15 (variant 0 of the plan is the
+// split-axis step, ksplit.cuh; entry 0 here is the plan's last variant and serves workspaces too small for
+// the split-axis step).  Entries, the plan's variants from 1 on: 0 column and velocity
 // passes on the 12 x 15 factorisation, density passes on 15 x 12 (fewer registers where the
 // state is preloaded), and 8-column tiles for the column passes of the forward sweep, which
 // runs alone on the GPU; 1 all 12 x 15, 4 rows / 4 columns per CTA; 2 the same with 8 rows /
