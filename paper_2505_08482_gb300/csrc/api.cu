@@ -13,18 +13,61 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <map>
+#include <mutex>
+#include <vector>
 
 #include "pat_internal.h"
 #include "vec.h"
 
 using namespace pat;
 
-float pat::scale_g(const pat_plan_s* p) {
-    return float(p->g.dt / p->g.rho0 / (double(p->ng) * p->ng) * std::pow(1.0 + p->gain, -2.0));
+// Mean gain of a forward and inverse transform pair of the generic passes minus 1, over the modes up to an eighth of the
+// sampling rate: with the transforms' float constants in FP64, once per process and side (5 ms at Ng 400).  It is not
+// that of the register transforms: Ng 180 2.0e-8, where those have -0.7e-8.
+static double generic_gain(const FftDesc& fd) {
+    static std::mutex mu;
+    static std::map<int, double> known;
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(fd.n);
+    if (it != known.end()) return it->second;
+    const int n = fd.n, top = n / 8;
+    std::vector<double2> e(n), a(n), b(n);
+    std::vector<float2> tw(n);
+    for (int q = 0; q < n; ++q) {
+        const double w = -2.0 * 3.14159265358979323846 * q / n;
+        e[q] = double2{std::cos(w), -std::sin(w)};
+        tw[q] = make_float2(float(std::cos(w)), float(std::sin(w)));
+    }
+    double mean = 0.0;
+    for (int k = -top; k <= top; ++k) {
+        auto mode = [&](int q) { return e[size_t((k + n) % n) * q % n]; };
+        for (int q = 0; q < n; ++q) a[q] = mode(q);
+        double2* x = fft_host<false>(a.data(), b.data(), fd, tw.data());
+        x = fft_host<true>(x, x == a.data() ? b.data() : a.data(), fd, tw.data());
+        double s = 0.0;
+        for (int q = 0; q < n; ++q) s += mode(q).x * x[q].x + mode(q).y * x[q].y;
+        mean += (s / (double(n) * n) - 1.0) / (2 * top + 1);
+    }
+    return known[n] = mean;
 }
-float pat::scale_d(const pat_plan_s* p) {
-    const double n2 = double(p->ng) * p->ng, target = p->g.dt / n2 * (p->g.dt / n2) * std::pow(1.0 + p->gain, -4.0);
-    return float(target / double(scale_g(p)));
+
+// (a gain of 0: the side has no compiled transforms, and its factors are not corrected)
+static double gain_of(const pat_plan_s* p, bool generic) {
+    if (!generic || p->gain == 0.0) return p->gain;
+    try {
+        return generic_gain(p->fft);
+    } catch (...) {   // no host memory: no exception leaves a C entry point
+        return 0.0;
+    }
+}
+float pat::scale_g(const pat_plan_s* p, bool generic) {
+    return float(p->g.dt / p->g.rho0 / (double(p->ng) * p->ng) * std::pow(1.0 + gain_of(p, generic), -2.0));
+}
+float pat::scale_d(const pat_plan_s* p, bool generic) {
+    const double n2 = double(p->ng) * p->ng,
+                 target = p->g.dt / n2 * (p->g.dt / n2) * std::pow(1.0 + gain_of(p, generic), -4.0);
+    return float(target / double(scale_g(p, generic)));
 }
 
 namespace {
@@ -38,9 +81,9 @@ namespace {
 // one forward step n -> n+1 given the row spectrum of p^n in A
 int step(const Launch& L, const Ws& w, int n, float* y, float* hist, int hist_slot) {
     const pat_plan_s* p = L.p;
-    RC(launch_col(L, w.A, w.B, 0, 0, scale_g(p)));
+    RC(launch_col(L, w.A, w.B, 0, 0, scale_g(p, !p->fast)));
     RC(launch_row_u(L, w, n == 0));
-    RC(launch_col(L, w.A, w.B, 1, 1, scale_d(p)));
+    RC(launch_col(L, w.A, w.B, 1, 1, scale_d(p, !p->fast)));
     RC(launch_row_rho(L, w, 0, nullptr, y, n + 1, hist, hist_slot));
     return PAT_OK;
 }
@@ -156,7 +199,7 @@ int reverse_sweep(pat_plan_s* p, const float* p0, const float* r, float* grad_p0
         PAT_CUDA(cudaMemsetAsync(w.ubx, 0, 4 * f * sizeof(float), st));
     }
     PAT_CUDA(cudaMemsetAsync(w.cbar, 0, size_t(p->K) * p->n * p->n * sizeof(float), st));
-    const float sg = scale_d(p), sd = scale_g(p);   // dt rho0 G t, dt/rho0 D t'
+    const float sg = scale_d(p, !p->fast), sd = scale_g(p, !p->fast);   // dt rho0 G t, dt/rho0 D t'
     cudaStream_t R = p->side;
     const int last = p->nseg - 1;
     // the side stream starts after everything issued so far on st (forward sweep, residual)

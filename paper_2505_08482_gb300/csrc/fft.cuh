@@ -184,4 +184,37 @@ __device__ float2* fft_smem(float2* a, float2* b, int nseq, int ss, const FftDes
     return a;
 }
 
+// One stage of stockham_stage for one sequence on the host, in FP64 arithmetic with the same float constants.
+template <int R, bool INV>
+inline void stockham_stage_host(const double2* src, double2* dst, int n, int Ns, const float2* tw) {
+    const int nb = n / R, tstride = n / (Ns * R);
+    for (int j = 0; j < nb; ++j) {
+        const int k = j % Ns;
+        double2 v[R];
+        for (int r = 0; r < R; ++r) {
+            v[r] = src[j + r * nb];
+            if (r > 0 && Ns > 1) v[r] = INV ? cmulc(v[r], tw[r * k * tstride]) : cmul(v[r], tw[r * k * tstride]);
+        }
+        dft_small<R, INV>(v);
+        for (int r = 0; r < R; ++r) dst[(j - k) * R + k + r * Ns] = v[r];
+    }
+}
+template <bool INV>
+inline double2* fft_host(double2* a, double2* b, const FftDesc& fd, const float2* tw) {
+    int Ns = 1;
+    for (int st = 0; st < fd.nrad; ++st) {
+        switch (fd.rad[st]) {
+            case 2: stockham_stage_host<2, INV>(a, b, fd.n, Ns, tw); break;
+            case 3: stockham_stage_host<3, INV>(a, b, fd.n, Ns, tw); break;
+            case 4: stockham_stage_host<4, INV>(a, b, fd.n, Ns, tw); break;
+            default: stockham_stage_host<5, INV>(a, b, fd.n, Ns, tw); break;
+        }
+        double2* t = a;
+        a = b;
+        b = t;
+        Ns *= fd.rad[st];
+    }
+    return a;
+}
+
 }  // namespace pat

@@ -660,8 +660,8 @@ int launch_forward_cluster(const Launch& L, const Ws& w, const float* p0, const 
     a.n0 = n0;
     a.n1 = n1;
     a.init = state ? 0 : 1;
-    a.sg = scale_g(p);
-    a.sd = scale_d(p);
+    a.sg = scale_g(p, false);
+    a.sd = scale_d(p, false);
     count_launch();
     int rc = p->clops->forward(geo_ws(p, w), L.st, a);
     if (rc != PAT_OK) return rc;
@@ -689,8 +689,8 @@ int launch_forward_persistent(const Launch& L, const Ws& w, const float* p0, flo
     a.last0 = last0;
     a.ckpt = ckpt;
     a.s = p->s_eff;
-    a.sg = scale_g(p);
-    a.sd = scale_d(p);
+    a.sg = scale_g(p, false);
+    a.sd = scale_d(p, false);
     a.nsteps = p->nt - 1;
     a.queue = w.queue;
     a.wait_ns = kQueueWaitNs;

@@ -113,7 +113,7 @@ struct pat_plan_s {
     const void* hist_valid_ws;
     int device;
     int sms;           // SMs of the device
-    double gain;       // mean gain of a float transform pair over the well-resolved modes (0: not measured)
+    double gain;       // mean gain of a register transform pair over the well-resolved modes (0: not measured)
     // captured CUDA graphs of whole calls, keyed by call kind, buffers and variant;
     // at most kMaxGraphs are kept, the least recently replayed one is dropped first
     static constexpr size_t kMaxGraphs = 16;
@@ -217,8 +217,9 @@ int split_configure(const SplitOps* ops);
 // dt/rho0 G and dt rho0 D of the four-pass step with the inverse 2-D FFT normalisation folded in, corrected for the
 // mean gain of the float transforms (two pairs in each); the second factor also makes
 // up for the rounding of the first, since their product sets the speed of sound.
-float scale_g(const pat_plan_s* p);
-float scale_d(const pat_plan_s* p);
+// generic: by the generic passes' transforms, else by the register transforms.
+float scale_g(const pat_plan_s* p, bool generic);
+float scale_d(const pat_plan_s* p, bool generic);
 // Forward sweep into y [K][nt][m] with workspace regions w (checkpoints kept if keep).
 int forward_sweep(pat_plan_s* p, const float* c, const float* p0, float* y, const Ws& w, bool keep,
                   cudaStream_t st);
