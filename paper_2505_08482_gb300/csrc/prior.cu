@@ -230,11 +230,11 @@ __device__ void scalar_step(const ScalarArgs& a) {   // all threads of one block
 
 // Dot products <a, b> per field into part, then (mode >= 0) the scalar step that uses them, by the block that is
 // done last: the sums keep their fixed order.  With z (CG update) first z += alpha d, r -= alpha q, and the product is
-// <r, r>.  grid (kDotBlocks, nf).
+// <r, r>.  grid (kDotBlocks, nf).  (part is no restricted pointer: the last block reads the same sums through sa.part.)
 __global__ void __launch_bounds__(256) k_pr_dot(const float* __restrict__ a, const float* __restrict__ b,
                                                 float* __restrict__ z, float* __restrict__ r,
                                                 const float* __restrict__ d, const float* __restrict__ q, size_t nn,
-                                                double* __restrict__ part, unsigned* __restrict__ done, ScalarArgs sa) {
+                                                double* part, unsigned* __restrict__ done, ScalarArgs sa) {
     __shared__ double red[256];
     __shared__ bool last;
     pdl_wait_then_release();
