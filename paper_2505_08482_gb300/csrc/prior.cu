@@ -49,7 +49,6 @@ struct pat_prior_s {
     unsigned* done = nullptr; // [1] blocks of the running dot product that are done (0 between launches)
     int sms = 1;
     int rows_per_cta, cols_per_cta;
-    size_t smem_rows, smem_cols;
 };
 
 namespace {
@@ -444,8 +443,6 @@ extern "C" int pat_prior_create(int n, double dx, double tau, int max_fields, pa
         cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
     p->rows_per_cta = 4;
     p->cols_per_cta = 8;
-    p->smem_rows = size_t(M + 2 * p->rows_per_cta * M) * sizeof(float2);
-    p->smem_cols = size_t(M + 2 * p->cols_per_cta * (M + 1)) * sizeof(float2);
     std::vector<float> hl(size_t(M) * M), hi(size_t(M) * M);
     for (size_t i = 0; i < hl.size(); ++i) {
         hl[i] = float(lam[i]);
@@ -480,11 +477,10 @@ extern "C" int pat_prior_create(int n, double dx, double tau, int max_fields, pa
     // copies from pageable memory may still be in flight when cudaMemcpy returns, and the
     // caller's non-blocking streams are not ordered after the legacy stream: wait for them
     if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-    const void* kerns[] = {(const void*)k_pr_rows_fwd, (const void*)k_pr_rows_inv};
-    for (const void* f : kerns)
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(p->smem_rows));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute((const void*)k_pr_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, int(p->smem_cols));
+    // The limit belongs to the kernel, not to the prior, and a smaller prior must not lower it below what a larger one
+    // launches with: the most a CTA can have.
+    for (const void* f : {(const void*)k_pr_rows_fwd, (const void*)k_pr_rows_inv, (const void*)k_pr_cols})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) {
         pat_prior_destroy(p);
         return cuda_fail(e, "pat_prior_create");
