@@ -237,14 +237,14 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-def stored_traffic(cls: int, src_hash: str, key: str = "dram_bytes_per_launch_full"):
+def stored_traffic(cls: int, src_hash: str, key: str = "dram_bytes_per_launch_full", phase: str = ""):
     """Per-launch DRAM bytes (or another per-launch ncu figure) of kernel class cls from the
-    committed ncu summary, if current."""
+    committed ncu summary, if current; phase: "forward" or "adjoint", for the classes that run in both."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
     d = json.load(open(p))
-    e = d.get(str(cls))
+    e = d.get(f"{cls} {phase}") or d.get(str(cls))
     if not e or d.get("kernel_source_hash") != src_hash:
         return None
     return e.get(key)
@@ -618,7 +618,7 @@ def run_ours(args, rank, world, local_rank):
     # the same launches against the instruction-issue peak (4 schedulers per SM, one warp
     # instruction per cycle each, at the maximum SM clock), from the warp instructions per launch
     # of the committed ncu capture
-    insts = stored_traffic(dom, src_hash, "warp_instructions_per_launch")
+    insts = stored_traffic(dom, src_hash, "warp_instructions_per_launch", dom_phase)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     sm_max = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("sm_max_mhz", 2070.0)) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 2070.0
@@ -629,7 +629,7 @@ def run_ours(args, rank, world, local_rank):
         "peak_kind": f"4 schedulers x {sms} SMs x {sm_max:.0f} MHz (one warp instruction per cycle each)",
         "source": "smsp__inst_executed.sum of the dominant pass (ncu, profiles/traffic.json)"}
     roof = {"bound": "hbm", "kernel": f"{B.KERNEL_CLASSES[dom]} ({dom_phase} sweep)", "achieved": achieved,
-            "peak": peak, "unit": "GB/s", "frac": achieved / peak, "traffic": stored_traffic(dom, src_hash),
+            "peak": peak, "unit": "GB/s", "frac": achieved / peak, "traffic": stored_traffic(dom, src_hash, phase=dom_phase),
             "peak_kind": f"{peak_kind} hbm_gbs (burst copy)", "algorithmic_bytes_per_launch": bpl,
             "avg_launch_us": dom_us, "launches_timed": dom_cnt,
             "timing": "every launch of the class bracketed by CUDA events on its stream in an eager sweep that "
