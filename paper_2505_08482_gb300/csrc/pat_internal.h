@@ -198,8 +198,8 @@ int launch_forward_cluster(const Launch& L, const Ws& w, const float* p0, const 
 // ---- split-axis passes (split.cu) ----
 // the initial pass from p0: rho lines, pressure lines, samples of level 0 (y, hist may be null)
 int split_start(const Launch& L, const Ws& w, const float* p0, float* y, float* hist, int hist_slot);
-// re-enter at a level from the real state [4][K][ng][ng] (u_x, u_y, rho_x, rho_y): lines of u and rho
-// (after_copy: the state may have been written by a copy), then the samples and pressure lines of that level
+// re-enter at a level from the real state [4][K][ng][ng] (u_x, u_y, rho_x, rho_y): lines of u and rho, then
+// the samples and pressure lines of that level
 int split_enter(const Launch& L, const Ws& w, const float* state, int level, float* y, float* hist, int hist_slot);
 // forward steps n0 .. n1-1; p^{n+1} into slot n+1-hbase of hist when hist and n+1 >= hbase; ckpt (or
 // null): the real state at every level that is a multiple of s, from which the sweep itself goes on,
