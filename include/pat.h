@@ -225,9 +225,10 @@ int pat_pml_auto(int n, int min_pml);
  * only is accepted by every call that takes a workspace, and the call then
  * runs the four-pass step (variant 0: the plan's last variant; else the generic
  * passes): with F = 4 K Ng^2 and S = 8 K Ng P bytes (P: Ng / 2 + 1 rounded up to
- * a multiple of 4) its state is 4 F + 2 S, in PAT_WS_GRADIENT twice, instead of
- * 24 K Ng (Ng + 2) + 2 F (each array rounded up to 256 bytes).  Such a gradient
- * workspace has its checkpoints where the larger one has them. */
+ * a multiple of 4) its state is 4 F + 2 S instead of 24 K Ng (Ng + 2) + 2 F, and
+ * twice that with the adjoint's (each array rounded up to 256 bytes).
+ * Checkpoints lie at the same place in a gradient workspace of either size, and
+ * calls that use it as a forward workspace leave them alone. */
 #define PAT_WS_FORWARD 0
 #define PAT_WS_GRADIENT 1
 size_t pat_workspace_bytes(pat_plan plan, int kind);

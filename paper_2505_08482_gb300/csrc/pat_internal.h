@@ -105,10 +105,10 @@ struct pat_plan_s {
     size_t ws_fwd, ws_grad;
     size_t ws_fwd_passes, ws_grad_passes;   // workspaces of the four-pass step alone
     // layout offsets (bytes): in a workspace, and within the state of a step
-    size_t o_state, o_state_grad, o_cg, o_J, o_part, o_flag, o_queue;
-    size_t o_ckpt, o_hist, o_cbar, o_resid, o_ypred;
-    size_t s_A, s_B, s_passes;          // four-pass step: spectra, size
-    size_t s_lr, s_la, s_re, s_most;    // split-axis passes: lines of rho and the pressure, real fields; larger size
+    size_t o_state, o_cg, o_J, o_part, o_flag, o_queue;
+    size_t o_ckpt, o_hist, o_cbar, o_resid, o_ypred, o_lub, o_lrb, o_la2, o_re2;
+    size_t s_A, s_B, s_passes;   // four-pass step: spectra, size
+    size_t s_lr, s_la, s_re;     // split-axis passes: lines of rho and the pressure, real fields
     // host bookkeeping: the workspace whose history holds the last segment
     const void* hist_valid_ws;
     int device;

@@ -89,7 +89,7 @@ Ws resolve(const pat_plan_s* p, void* base, size_t bytes, bool grad) {
     auto four = [f](char* at, float* (&v)[4]) {
         for (int i = 0; i < 4; ++i) v[i] = reinterpret_cast<float*>(at) + i * f;
     };
-    char* st = b + (grad ? p->o_state_grad : p->o_state);
+    char* st = b + p->o_state;
     float* v[4];
     four(st, v);
     w.ux = v[0]; w.uy = v[1]; w.rx = v[2]; w.ry = v[3];
@@ -100,42 +100,42 @@ Ws resolve(const pat_plan_s* p, void* base, size_t bytes, bool grad) {
     w.la = reinterpret_cast<float2*>(st + p->s_la);
     w.re = reinterpret_cast<float*>(st + p->s_re);
     if (grad) {
+        char* ad = st + p->s_passes;
+        four(ad, v);
+        w.ubx = v[0]; w.uby = v[1]; w.rbx = v[2]; w.rby = v[3];
+        w.A2 = reinterpret_cast<float2*>(ad + p->s_A);
+        w.B2 = reinterpret_cast<float2*>(ad + p->s_B);
         w.ckpt = reinterpret_cast<float*>(b + p->o_ckpt);
         w.hist = reinterpret_cast<float*>(b + p->o_hist);
         w.cbar = reinterpret_cast<float*>(b + p->o_cbar);
         w.resid = reinterpret_cast<float*>(b + p->o_resid);
         w.ypred = reinterpret_cast<float*>(b + p->o_ypred);
-        // the adjoint state: the same regions again behind the forward state
-        char* ad = st + (w.split_fits ? p->s_most : p->s_passes);
-        four(ad, v);
-        w.ubx = v[0]; w.uby = v[1]; w.rbx = v[2]; w.rby = v[3];
-        w.A2 = reinterpret_cast<float2*>(ad + p->s_A);
-        w.B2 = reinterpret_cast<float2*>(ad + p->s_B);
-        w.lub = reinterpret_cast<float2*>(ad);
-        w.lrb = reinterpret_cast<float2*>(ad + p->s_lr);
-        w.la2 = reinterpret_cast<float2*>(ad + p->s_la);
-        w.re2 = reinterpret_cast<float*>(ad + p->s_re);
+        w.lub = reinterpret_cast<float2*>(b + p->o_lub);
+        w.lrb = reinterpret_cast<float2*>(b + p->o_lrb);
+        w.la2 = reinterpret_cast<float2*>(b + p->o_la2);
+        w.re2 = reinterpret_cast<float*>(b + p->o_re2);
     }
     return w;
 }
 
-// What outlives a call (checkpoints, history, status) comes first; the state of a step follows, the four-pass step's
-// and the split-axis passes' over the same memory (a call runs one of them; checkpoints and the pressure history are
-// real fields in both).  A workspace that holds the four-pass step only is laid out alike up to that state, so that
-// calls with workspaces of either size share checkpoints.
+// A workspace: medium, sums and status; the state of a step; checkpoints, history and what else a gradient keeps for a call.
+// The four-pass step's state, forward and adjoint, and the split-axis passes' lie over the same memory (a call runs one of
+// them; checkpoints and the pressure history are real fields in both).  A forward workspace ends within the two, so that
+// forward calls in a gradient workspace leave its checkpoints alone, and all offsets are those of the workspace that holds
+// the four-pass step only, so that calls with workspaces of either size share checkpoints.  What of the split-axis
+// passes' adjoint does not fit beside their forward state comes last.
 static void layout(pat_plan_s* p) {
     const size_t f = size_t(p->K) * p->ng * p->ng * sizeof(float);
     const size_t spec = size_t(p->K) * p->ng * p->hp * sizeof(float2);
-    const size_t lines = 2 * size_t(p->K) * p->hc * p->ng * sizeof(float2);
-    size_t q = align256(4 * f);   // four-pass: state, two spectra
-    p->s_A = q; q = align256(q + spec);
-    p->s_B = q; q = align256(q + spec);
-    p->s_passes = p->s_most = q;
-    q = align256(lines);          // split-axis: lines of u, rho and the pressure, two real fields
-    p->s_lr = q; q = align256(q + lines);
-    p->s_la = q; q = align256(q + lines);
-    p->s_re = q; q = align256(q + 2 * f);
-    if (split_ops_for(p->ng)) p->s_most = std::max(p->s_passes, q);
+    const size_t lines = align256(2 * size_t(p->K) * p->hc * p->ng * sizeof(float2));
+    const bool split = split_ops_for(p->ng) != nullptr;
+    p->s_A = align256(4 * f);   // four-pass: state, two spectra
+    p->s_B = p->s_A + align256(spec);
+    p->s_passes = p->s_B + align256(spec);
+    p->s_lr = lines;            // split-axis: lines of u, rho and the pressure, two real fields
+    p->s_la = 2 * lines;
+    p->s_re = 3 * lines;
+    const size_t s_split = split ? 3 * lines + align256(2 * f) : 0;
     size_t o = 0;
     p->o_cg = o; o = align256(o + size_t(p->ninst) * p->ng * p->ng * sizeof(float));
     p->o_J = o; o = align256(o + size_t(p->ninst) * sizeof(double));
@@ -144,16 +144,30 @@ static void layout(pat_plan_s* p) {
     p->o_queue = o; o = align256(o + (size_t(p->K) + 2) * sizeof(int));
     p->o_state = o;
     p->ws_fwd_passes = o + p->s_passes;
-    p->ws_fwd = o + p->s_most;
+    p->ws_fwd = o + std::max(p->s_passes, s_split);   // (s_split < 2 s_passes on every side)
+    const size_t kept = o + 2 * p->s_passes;
+    o = kept;
     p->o_ckpt = o; o = align256(o + size_t(std::max(p->nseg - 1, 0)) * 4 * f);
     p->o_hist = o; o = align256(o + size_t(p->nseg > 1 ? 2 : 1) * p->K * p->s_eff * p->ng * p->ng * sizeof(float));
     p->o_cbar = o; o = align256(o + size_t(p->K) * p->n * p->n * sizeof(float));
     const size_t tr = size_t(p->K) * p->nt * p->m * sizeof(float);
     p->o_resid = o; o = align256(o + tr);
     p->o_ypred = o; o = align256(o + tr);
-    p->o_state_grad = o;
-    p->ws_grad_passes = o + 2 * p->s_passes;
-    p->ws_grad = o + 2 * p->s_most;
+    p->ws_grad_passes = o;
+    size_t q = p->o_state + s_split;
+    auto place = [&](size_t* at, size_t bytes) {
+        size_t& end = q + bytes <= kept ? q : o;
+        *at = end;
+        end += bytes;
+    };
+    p->o_lub = p->o_lrb = p->o_la2 = p->o_re2 = 0;
+    if (split) {
+        place(&p->o_lub, lines);
+        place(&p->o_re2, align256(2 * f));
+        place(&p->o_lrb, lines);
+        place(&p->o_la2, lines);
+    }
+    p->ws_grad = o;
 }
 
 }  // namespace pat

@@ -132,3 +132,30 @@ def test_autotune_in_a_four_pass_workspace(ng):
             assert np.isinf(ms[1]) and plan.variant != 0 and ms[plan.variant + 1] == min(ms)
         else:
             assert plan.variant == -1
+
+
+@pytest.mark.parametrize("ng,s", [(108, 7), (80, 6), (150, 5), (60, 7)])
+def test_forward_calls_leave_the_checkpoints_alone(ng, s):
+    """A forward-size call in a gradient workspace (either size) between the kept forward pass and vjp."""
+    from paper_2505_08482_gb300 import _binding as B
+    n, K, nt, M = ng - 40, 2, 24, 9
+    rng = ps.rng_for(ng)
+    c = _dev(ps.ellipse_phantom(n, 3, rng))
+    p0 = _dev(np.stack([ps.blob_p0(n, 4, rng, sigma_cells=(2.0, 5.0)) for _ in range(K)]))
+    xy = ps.rng_for(ng + 1).uniform(0.2 * n, 0.8 * n, size=(M, 2)) * 1e-4
+    plan = gpu_plan(grid_params(n, nt, pml=20), xy, K, ckpt_every=s)
+    assert plan.ng == ng
+    fwd, grad = _four_pass_bytes(ng, n, K, 1, nt, M, s)
+    full_f, full_g = plan.workspace_bytes(B.PAT_WS_FORWARD), plan.workspace_bytes(B.PAT_WS_GRADIENT)
+    yb = torch.randn((K, nt, M), device="cuda", generator=torch.Generator(device="cuda").manual_seed(2))
+    k = _Calls(plan, full_g)
+    for size in (full_g, grad):
+        assert k.forward(c, p0, size)[0] == B.PAT_OK
+        assert k.vjp(c, p0, yb, size)[0] == B.PAT_OK
+        rc, gp, gc = k.vjp(c, p0, yb, size)          # every segment recomputed
+        assert rc == B.PAT_OK and float(gc.abs().max()) > 0
+        for between in (fwd, full_f):
+            assert k.forward(c, p0, size)[0] == B.PAT_OK
+            assert k.forward(c, 2.0 * p0, between)[0] == B.PAT_OK
+            rc, a, b = k.vjp(c, p0, yb, size)
+            assert rc == B.PAT_OK and torch.equal(a, gp) and torch.equal(b, gc), (size, between)
